@@ -22,6 +22,7 @@
 
 #include "../../include/hss.h"
 #include "common.cuh"
+#include "fxgemm.cuh"
 #include "ulv_kernels.cuh"
 #include "uneven.cuh"
 
@@ -177,8 +178,8 @@ size_t layout(hss_batch_s* bt, char* base) {
 void gemm(bool ta, bool tb, int m, int n, int k, double alpha, const double* A, int lda,
           long long sA, const double* B, int ldb, long long sB, double beta, double* C, int ldc,
           long long sC, long long batch, cudaStream_t st) {
-  if (batch > 0) gemm_batched<double>(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc,
-                                      sC, (int)batch, st);
+  if (batch > 0)
+    dgemm_batched(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, (int)batch, st);
 }
 
 #define TRY(call)                                                                      \
@@ -241,7 +242,7 @@ int factor_group(hss_batch_s* bt, Group& g) {
     gemm(true, false, r, r, b, 1.0, t.V, b, br, g.Y, b, br, 0.0, g.X, r, rr, n, st);
     gemm(true, false, r, r, r, 1.0, t.T, r, rr, g.X, r, rr, 0.0, g.Z, r, rr, n, st);
     gemm(false, false, b, r, r, -0.5, t.V, b, br, g.Z, r, rr, 1.0, g.Y, b, br, n, st);
-    syr2k_lower_batched<double>(b, r, Ain, b, bb, g.Y, b, br, t.V, b, br, t.M, b, bb, (int)n, st);
+    dsyr2k_lower_batched(b, r, Ain, b, bb, g.Y, b, br, t.V, b, br, t.M, b, bb, (int)n, st);
     if (t.split > 0)
       TRY(launch_pchol<double>(t.M, b, bb, b, c, g.ht[h + 1].A, 2 * r, 4 * rr, t.ldp, h, 0,
                                bt->status, (int)t.split, st));

@@ -19,6 +19,7 @@
 #include "basis.cuh"
 #include "common.cuh"
 #include "dfgemm.cuh"
+#include "fxgemm.cuh"
 #include "ir_kernels.cuh"
 #include "tc_gemm.cuh"
 #include "ulv_kernels.cuh"
@@ -382,7 +383,33 @@ void gemm(hss_s* h, bool ta, bool tb, int m, int n, int k, T alpha, const T* A, 
   if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return;
   Launch l(h, n <= 32 ? HSS_K_GEMM_SKINNY : HSS_K_GEMM, 2.0 * m * n * (double)k * batch, st,
            sizeof(T) == 4);
-  gemm_batched<T>(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, st);
+  if constexpr (std::is_same<T, double>::value)
+    dgemm_batched(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, st);
+  else
+    gemm_batched<T>(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, st);
+}
+
+// A - P Qᵀ - Q Pᵀ and A - P Pᵀ on the lower triangle, the latter with the merge
+// into the parents' blocks PA where given
+template <typename T>
+void syr2k(int m, int k, const T* A, int lda, long long sA, const T* P, int ldp, long long sP,
+           const T* Q, int ldq, long long sQ, T* M, int ldm, long long sM, int batch,
+           cudaStream_t st) {
+  if constexpr (std::is_same<T, double>::value)
+    dsyr2k_lower_batched(m, k, A, lda, sA, P, ldp, sP, Q, ldq, sQ, M, ldm, sM, batch, st);
+  else
+    syr2k_lower_batched<T>(m, k, A, lda, sA, P, ldp, sP, Q, ldq, sQ, M, ldm, sM, batch, st);
+}
+
+template <typename T>
+void syrk(int m, int k, const T* A, int lda, long long sA, const T* P, int ldp, long long sP, T* M,
+          int ldm, long long sM, T* PA, int ldpa, long long sPA, int batch, cudaStream_t st) {
+  if constexpr (std::is_same<T, double>::value)
+    dsyrk_lower_batched(m, k, A, lda, sA, P, ldp, sP, M, ldm, sM, PA, ldpa, sPA, batch, st);
+  else if (PA)
+    syrk_lower_merge_batched<T>(m, k, A, lda, sA, P, ldp, sP, M, ldm, sM, PA, ldpa, sPA, batch, st);
+  else
+    syrk_lower_batched<T>(m, k, A, lda, sA, P, ldp, sP, M, ldm, sM, batch, st);
 }
 
 // partial Cholesky of the first c of b columns: POTRF c x c, TRSM (b-c) x c,
@@ -508,7 +535,7 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
       }
     } else {
       Launch k(h, HSS_K_SYR2K, 2.0 * r * b * (b + 1.0) * n, st, sizeof(T) == 4);
-      syr2k_lower_batched<T>(b, r, Ain, b, bb, f.Y, b, br, P.V, b, br, P.M, b, bb, n, st);
+      syr2k<T>(b, r, Ain, b, bb, f.Y, b, br, P.V, b, br, P.M, b, bb, n, st);
     }
     // (c) partial Cholesky of the first c columns, blocked over the whole level:
     // per panel of kPanel columns a per-node panel kernel (diagonal block and
@@ -527,11 +554,9 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
       if (nt > 0) {
         Launch k(h, HSS_K_SYR2K, (double)nt * (nt + 1.0) * kb * n, st, sizeof(T) == 4);
         T* Tr = Mk + kb + (long long)kb * b;
-        if (k0 + kb == c)   // the last update leaves Â^SS: its epilogue is the merge
-          syrk_lower_merge_batched<T>(nt, kb, Tr, b, bb, Mk + kb, b, bb, Tr, b, bb, Q.A, ldq, sq,
-                                      n, st);
-        else
-          syrk_lower_batched<T>(nt, kb, Tr, b, bb, Mk + kb, b, bb, Tr, b, bb, n, st);
+        // the last update leaves Â^SS: its epilogue is the merge
+        syrk<T>(nt, kb, Tr, b, bb, Mk + kb, b, bb, Tr, b, bb, k0 + kb == c ? Q.A : nullptr, ldq,
+                sq, n, st);
       }
     }
     // (d, second half) with nothing eliminated (c = 0) Â^SS is the whole block:

@@ -1,0 +1,476 @@
+// FP64 products on the tensor cores by exact slicing (the Ozaki scheme: Ozaki,
+// Ogita, Oishi, Rump 2012; on tensor cores Mukunoki, Ozaki, Ogita, Imamura 2020).
+//
+// The chip's FP64 pipe gives 1.05 TFLOP/s (2 DFMA per clock per SM); its FP16
+// MMA 600 TFLOP/s with FP32 accumulation, which is exact as long as every
+// partial sum is an integer of at most 24 bits.  Within a group of kGroup = 128
+// inner indices, each row of an operand is scaled by the power of two e of its
+// largest element and cut to a 64-bit integer q, |q| < 2^63; q is written as
+// eight digits of base 256 in [-128, 127] (exact in FP16), and of the 64 digit
+// products the 36 with weight i + j <= 7 are accumulated, those of equal weight
+// in one FP32 accumulator: at most 8 x 128 products of magnitude <= 2^14, a sum
+// of at most 2^24, so every MMA is exact.  At the end of a group the eight
+// accumulators are put together as two integers and added to the FP64 result.
+//
+// Error of one group: cutting each operand at 2^-63 of its row's largest
+// element, and the dropped digit products, about 2^-63 of max|a| max|b| a product:
+// far below the 2^-53 of a partial sum that each step of a DFMA chain rounds
+// off, also where a row's largest element dwarfs the others (seven digits, whose
+// error is 2^-56 of max|a| max|b|, are not enough there: the solves of kernel
+// matrices lost a factor of three to five against the DFMA chain).  Rows with an
+// element that is not finite or whose largest magnitude is outside
+// [2^-470, 2^470] take a DFMA loop instead, so that infinities, NaN and
+// overflow behave as in the plain product.
+//
+// Layout: a CTA has 4 warps and a 64 x BN tile of C (BN = 32, 16 or 8 columns;
+// a warp 16 rows and every column).  Per group the operands' strips are read
+// once for the row maxima and, from L1 or L2, again in chunks of 32 inner indices
+// for the conversion to digits in shared memory (80-byte rows: ldmatrix and
+// 16-byte stores without bank conflicts); 8 weights x BN / 2 FP32 accumulators
+// live in registers.  Several CTAs share an SM, one converting while another
+// issues MMAs.
+#include <stdint.h>
+
+#include <map>
+#include <mutex>
+#include <tuple>
+
+#include "common.cuh"
+#include "fxgemm.cuh"
+
+namespace {
+
+constexpr int kThreads = 128;
+constexpr int kRows = 64;       // rows of a CTA's tile
+constexpr int kChunk = 32;      // inner indices converted at a time
+constexpr int kGroup = 128;     // inner indices with one scale
+constexpr int kDigits = 8;
+constexpr int kPitch = 2 * kChunk + 16;   // bytes of a row of digits in shared memory
+constexpr int kHiBig = (1023 + 470) << 20, kHiSmall = (1023 - 470) << 20;
+
+struct FxShape {
+  int m, n, K, K1;   // K1: inner indices of each part, K in all
+  FxOperand a, b;
+  double alpha, beta;
+  const double* Cin;
+  int ldcin;
+  long long sCin;
+  double* C;
+  int ldc;
+  long long sC;
+  int lower;
+  double* PA;
+  int ldpa;
+  long long sPA;
+  int tiles_m, tiles_n, tiles;
+};
+
+HSS_DEVINL uint32_t smem_of(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+
+HSS_DEVINL uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) { return __byte_perm(a, b, sel); }
+
+// fp16x2 of two digits held as 1024 + (digit + 128): minus 1152
+HSS_DEVINL uint32_t unbias(uint32_t v) {
+  uint32_t r;
+  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(0x64806480u));
+  return r;
+}
+
+HSS_DEVINL uint32_t shr(uint32_t v, uint32_t n) {   // 0 for n >= 32
+  uint32_t r;
+  asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+  return r;
+}
+
+// v 2^(63 - e), cut to an integer, + 0x8080808080808080: its bytes are the digits
+// plus 128, least significant first; E1 = e + 1023, e + 1022 the row's biased
+// exponent.  The mantissa, its leading one at bit 63, is shifted right and
+// negated with the sign; zeros and denormals (exponent field 0) are shifted out.
+HSS_DEVINL uint64_t fixed_point(double v, int E1) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  const uint32_t n = (uint32_t)(E1 - (int)((hi >> 20) & 0x7ffu));
+  const uint32_t top = __funnelshift_l(lo, hi, 11) | 0x80000000u;
+  const uint32_t tl = shr(__funnelshift_rc(lo << 11, top, n), (uint32_t)max((int)n - 32, 0));
+  const uint32_t th = shr(top, n);
+  const uint32_t s = (uint32_t)((int)hi >> 31);
+  return (((uint64_t)(th ^ s) << 32) | (tl ^ s)) +
+         ((0x80808080ull << 32) | (uint64_t)(0x80808080u - s));
+}
+
+// digit pairs of the elements u0 (lower half) and u1, most significant first
+HSS_DEVINL void digits(uint64_t u0, uint64_t u1, uint32_t (&d)[kDigits]) {
+  const uint32_t w0[2] = {(uint32_t)(u0 >> 32), (uint32_t)u0},
+                 w1[2] = {(uint32_t)(u1 >> 32), (uint32_t)u1};
+  const uint32_t c = 0x64646464u;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t up = prmt(w0[h], w1[h], 0x7362), dn = prmt(w0[h], w1[h], 0x5140);
+    d[4 * h + 0] = unbias(prmt(up, c, 0x4342));
+    d[4 * h + 1] = unbias(prmt(up, c, 0x4140));
+    d[4 * h + 2] = unbias(prmt(dn, c, 0x4342));
+    d[4 * h + 3] = unbias(prmt(dn, c, 0x4140));
+  }
+}
+
+HSS_DEVINL void ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+
+HSS_DEVINL void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// R rows (from row0 on) of one operand's part (contiguous inner indices 0 .. K-1
+// of one array).  Rows past the last are read as copies of it: their results are
+// not stored.
+template <int R, bool KC>
+struct Strip {
+  const double* p;   // KC: element (0, 0) of the operand; else the same
+  int ld, row0, last;
+
+  HSS_DEVINL const double* row(int r) const {
+    const int i = min(row0 + r, last);
+    return KC ? p + (long long)i * ld : p + i;
+  }
+  HSS_DEVINL double at(int r, int k) const { return row(r)[KC ? (long long)k : (long long)k * ld]; }
+
+  // mx[r] = largest high word (sign removed) of row r over [k0, k1); mx is cleared
+  HSS_DEVINL void maxima(int k0, int k1, int* mx) const {
+    const int tid = threadIdx.x;
+    if (KC) {
+      const int lane = tid & 31, w = tid >> 5;
+      constexpr int U = R / 4 < 4 ? R / 4 : 4;
+      for (int r = w; r < R; r += 4 * U) {
+        int v[U][kGroup / 32];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const double* q = row(r + 4 * u) + k0 + lane;
+#pragma unroll
+          for (int j = 0; j < kGroup / 32; ++j)
+            v[u][j] = k0 + lane + 32 * j < k1 ? __double2hiint(q[32 * j]) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          int h = 0;
+#pragma unroll
+          for (int j = 0; j < kGroup / 32; ++j) h = max(h, v[u][j] & 0x7fffffff);
+          h = __reduce_max_sync(0xffffffffu, h);
+          if (lane == 0) mx[r + 4 * u] = h;
+        }
+      }
+    } else {
+      constexpr int S = kThreads / R;   // threads per row
+      const int r = tid % R, n = k1 - k0;
+      int k = tid / R, h = 0;
+      const double* q = row(r) + (long long)(k0 + k) * ld;
+      const long long step = (long long)S * ld;
+      for (; k + 15 * S < n; k += 16 * S) {
+        int v[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j, q += step) v[j] = __double2hiint(*q);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) h = max(h, v[j] & 0x7fffffff);
+      }
+#pragma unroll 4
+      for (; k < n; k += S, q += step) h = max(h, __double2hiint(*q) & 0x7fffffff);
+      atomicMax(mx + r, h);
+    }
+  }
+
+  // digits of [k0, k0 + kChunk) (zero from k1 on) to shared memory, digit s of
+  // row r, index k at sm + s R kPitch + r kPitch + 2 (k - k0)
+  template <bool WHOLE>
+  HSS_DEVINL void convert(int k0, int k1, const int* E1, unsigned char* sm) const {
+    const int tid = threadIdx.x;
+    if (KC) {
+      constexpr int UNITS = R * kChunk / 2 / kThreads;   // (row, pair of k) per thread
+      double v[UNITS][2];
+      const int kp = 2 * (tid & 15);
+      // pairs past the end read the last pair's place
+      const bool ok0 = WHOLE || k0 + kp < k1, ok1 = WHOLE || k0 + kp + 1 < k1;
+#pragma unroll
+      for (int u = 0; u < UNITS; ++u) {
+        const double* q = row((tid >> 4) + 8 * u) + k0 + kp;
+        v[u][0] = ok0 ? q[0] : 0.0;
+        v[u][1] = ok1 ? q[1] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < UNITS; ++u) {
+        const int r = (tid >> 4) + 8 * u;
+        uint32_t d[kDigits];
+        digits(fixed_point(v[u][0], E1[r]), fixed_point(v[u][1], E1[r]), d);
+#pragma unroll
+        for (int s = 0; s < kDigits; ++s)
+          *reinterpret_cast<uint32_t*>(sm + (s * R + r) * kPitch + 2 * kp) = d[s];
+      }
+    } else {
+      for (int u = tid; u < 4 * R; u += kThreads) {   // (row, 8 consecutive k)
+        const int r = u % R, o = u / R;
+        double v[8];
+        const double* q = row(r) + (long long)(k0 + 8 * o) * ld;
+#pragma unroll
+        for (int j = 0; j < 8; ++j, q += ld) v[j] = (WHOLE || k0 + 8 * o + j < k1) ? *q : 0.0;
+        const int e = E1[r];
+        uint32_t d[4][kDigits];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          digits(fixed_point(v[2 * j], e), fixed_point(v[2 * j + 1], e), d[j]);
+#pragma unroll
+        for (int s = 0; s < kDigits; ++s)
+          *reinterpret_cast<uint4*>(sm + (s * R + r) * kPitch + 16 * o) =
+              make_uint4(d[0][s], d[1][s], d[2][s], d[3][s]);
+      }
+    }
+  }
+};
+
+template <int BN>
+constexpr int fx_smem() {
+  return kDigits * (kRows + BN) * kPitch;
+}
+
+template <int BN, bool AKC, bool BKC>
+__global__ void __launch_bounds__(kThreads, BN == 32 ? 2 : 3)
+fx_gemm_kernel(const __grid_constant__ FxShape s) {
+  constexpr int NB = BN / 8;
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ int ex[kRows + BN];   // row maxima, then the rows' exponents
+  unsigned char* smA = sm;
+  unsigned char* smB = sm + kDigits * kRows * kPitch;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const long long z = blockIdx.x / s.tiles;
+  int t = (int)(blockIdx.x % s.tiles), tm, tn;
+  if (s.lower) {   // row block tm has the column blocks that start at or left of its last row
+    tm = 0;
+    for (;; ++tm) {
+      const int have = min(s.tiles_n, (kRows * tm + kRows - 1) / BN + 1);
+      if (t < have) break;
+      t -= have;
+    }
+    tn = t;
+  } else {
+    tm = t % s.tiles_m;
+    tn = t / s.tiles_m;
+  }
+  const int i0 = tm * kRows, j0 = tn * BN;
+
+  float acc[kDigits][NB][4];
+  double res[NB][4];
+#pragma unroll
+  for (int b = 0; b < NB; ++b)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) res[b][e] = 0.0;
+
+  // parts of the inner index (two arrays per operand in the rank-2k update)
+  for (int part = 0; part * s.K1 < s.K; ++part) {
+  const Strip<kRows, AKC> A{(part ? s.a.p2 : s.a.p1) + z * (part ? s.a.s2 : s.a.s1),
+                            part ? s.a.ld2 : s.a.ld1, i0, s.m - 1};
+  const Strip<BN, BKC> B{(part ? s.b.p2 : s.b.p1) + z * (part ? s.b.s2 : s.b.s1),
+                         part ? s.b.ld2 : s.b.ld1, j0, s.n - 1};
+  for (int kg = 0; kg < s.K1; kg += kGroup) {
+    const int ke = min(s.K1, kg + kGroup);
+    for (int r = tid; r < kRows + BN; r += kThreads) ex[r] = 0;
+    __syncthreads();
+    A.maxima(kg, ke, ex);
+    B.maxima(kg, ke, ex + kRows);
+    __syncthreads();
+    int odd = 0;
+    for (int r = tid; r < kRows + BN; r += kThreads) {
+      const int h = ex[r];
+      odd |= h >= kHiBig || (h > 0 && h < kHiSmall);
+      // |v| < 0.996 2^(E - 1022): a mantissa near 2 goes up to the next power,
+      // so that the digits' range holds it
+      ex[r] = (h ? (h + 0x2100) >> 20 : 1023) + 1;
+    }
+    if (__syncthreads_or(odd)) {   // plain FP64 for this group
+      for (int k = kg; k < ke; ++k)
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int r = w * 16 + (lane >> 2) + 8 * (e >> 1);
+            const int c = 8 * b + 2 * (lane & 3) + (e & 1);
+            res[b][e] = fma(A.at(r, k), B.at(c, k), res[b][e]);
+          }
+      __syncthreads();
+      continue;
+    }
+#pragma unroll
+    for (int q = 0; q < kDigits; ++q)
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[q][b][e] = 0.f;
+    for (int kc = kg; kc < ke; kc += kChunk) {
+      if (kc + kChunk <= ke) {
+        A.template convert<true>(kc, ke, ex, smA);
+        B.template convert<true>(kc, ke, ex + kRows, smB);
+      } else {
+        A.template convert<false>(kc, ke, ex, smA);
+        B.template convert<false>(kc, ke, ex + kRows, smB);
+      }
+      __syncthreads();
+#pragma unroll 1
+      for (int ks = 0; ks < kChunk / 16; ++ks) {
+        if (kc + 16 * ks >= ke) break;
+        uint32_t a[kDigits][4];
+        const uint32_t aa =
+            smem_of(smA) + (w * 16 + (lane & 15)) * kPitch + ks * 32 + (lane >> 4) * 16;
+#pragma unroll
+        for (int q = 0; q < kDigits; ++q) ldmatrix4(a[q], aa + q * kRows * kPitch);
+        // two blocks of 8 columns per load (BN = 8: both halves of the 16 indices of one)
+        const uint32_t ba = smem_of(smB) + ks * 32 + ((lane >> 3) & 1) * 16 +
+                            ((lane & 7) + (NB > 1 ? (lane >> 4) << 3 : 0)) * kPitch;
+#pragma unroll
+        for (int b = 0; b < NB; b += 2)
+#pragma unroll
+          for (int j = 0; j < kDigits; ++j) {
+            uint32_t v[4];
+            ldmatrix4(v, ba + (j * BN + 8 * b) * kPitch);
+#pragma unroll
+            for (int i = 0; i + j < kDigits; ++i) {
+              mma_f16(acc[i + j][b], a[i], v[0], v[1]);
+              if (NB > 1) mma_f16(acc[i + j][b + (NB > 1)], a[i], v[2], v[3]);
+            }
+          }
+      }
+      __syncthreads();
+    }
+    // the group's sum: 2^(ea + eb - 70) (H 2^32 + L)
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        long long H = 0, L = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          H += (long long)__float2int_rn(acc[q][b][e]) * (1 << (24 - 8 * q));
+          L += (long long)__float2int_rn(acc[q + 4][b][e]) * (1 << (24 - 8 * q));
+        }
+        const int r = w * 16 + (lane >> 2) + 8 * (e >> 1);
+        const int c = 8 * b + 2 * (lane & 3) + (e & 1);
+        const double scale = __hiloint2double((ex[r] + ex[kRows + c] - 1093) << 20, 0);
+        res[b][e] = fma(fma((double)H, 4294967296.0, (double)L), scale, res[b][e]);
+      }
+    __syncthreads();
+  }
+  }
+
+  double* C = s.C + z * s.sC;
+  const double* Ci = s.Cin + z * s.sCin;
+#pragma unroll
+  for (int b = 0; b < NB; ++b)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int i = i0 + w * 16 + (lane >> 2) + 8 * (e >> 1);
+      const int j = j0 + 8 * b + 2 * (lane & 3) + (e & 1);
+      if (i >= s.m || j >= s.n || (s.lower && i < j)) continue;
+      double v = s.alpha * res[b][e];
+      if (s.beta != 0.0) v = fma(s.beta, Ci[i + (long long)j * s.ldcin], v);
+      C[i + (long long)j * s.ldc] = v;
+      if (s.PA) {
+        double* pa = s.PA + (z >> 1) * s.sPA;
+        const int off = (int)(z & 1) * s.m;
+        pa[(off + i) + (long long)(off + j) * s.ldpa] = v;
+        if (i != j) pa[(off + j) + (long long)(off + i) * s.ldpa] = v;
+      }
+    }
+}
+
+// dynamic shared memory above the default, once per device and kernel
+template <typename F>
+cudaError_t allow_smem(F kernel, int bytes) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, const void*>, cudaError_t> memo;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const auto key = std::make_tuple(dev, reinterpret_cast<const void*>(kernel));
+  std::lock_guard<std::mutex> g(mu);
+  const auto it = memo.find(key);
+  if (it != memo.end()) return it->second;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  memo[key] = e;
+  return e;
+}
+
+template <int BN, bool AKC, bool BKC>
+cudaError_t launch(FxShape& s, int batch, cudaStream_t st) {
+  s.tiles_m = (s.m + kRows - 1) / kRows;
+  s.tiles_n = (s.n + BN - 1) / BN;
+  s.tiles = s.tiles_m * s.tiles_n;
+  if (s.lower) {
+    s.tiles = 0;
+    for (int tm = 0; tm < s.tiles_m; ++tm) {
+      const int have = (kRows * tm + kRows - 1) / BN + 1;
+      s.tiles += have < s.tiles_n ? have : s.tiles_n;
+    }
+  }
+  const cudaError_t e = allow_smem(fx_gemm_kernel<BN, AKC, BKC>, fx_smem<BN>());
+  if (e != cudaSuccess) return e;
+  fx_gemm_kernel<BN, AKC, BKC>
+      <<<(unsigned)((long long)s.tiles * batch), kThreads, fx_smem<BN>(), st>>>(s);
+  return cudaGetLastError();
+}
+
+template <int BN>
+cudaError_t launch_modes(FxShape& s, int batch, cudaStream_t st) {
+  if (s.a.kc) return s.b.kc ? launch<BN, true, true>(s, batch, st) : launch<BN, true, false>(s, batch, st);
+  return s.b.kc ? launch<BN, false, true>(s, batch, st) : launch<BN, false, false>(s, batch, st);
+}
+
+}  // namespace
+
+cudaError_t fx_gemm(int m, int n, int K, const FxOperand& a, const FxOperand& b, double alpha,
+                    double beta, const double* Cin, int ldcin, long long sCin, double* C, int ldc,
+                    long long sC, int batch, bool lower, double* PA, int ldpa, long long sPA,
+                    cudaStream_t st) {
+  FxShape s{m, n, K, a.p2 ? K / 2 : K, a, b, alpha, beta, Cin ? Cin : C, ldcin, sCin, C, ldc, sC, lower ? 1 : 0,
+            PA, ldpa, sPA, 0, 0, 0};
+  if (n <= 8) return launch_modes<8>(s, batch, st);
+  if (n <= 16) return launch_modes<16>(s, batch, st);
+  return launch_modes<32>(s, batch, st);
+}
+
+void dgemm_batched(bool transA, bool transB, int m, int n, int k, double alpha, const double* A,
+                   int lda, long long sA, const double* B, int ldb, long long sB, double beta,
+                   double* C, int ldc, long long sC, int batch, cudaStream_t st) {
+  if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return;
+  // A few inner indices and columns on few rows (the tree of a rank <= 8 matrix):
+  // the FP64 pipe's kernels take 4.2 us against 6.2 us, whose digits are padded to
+  // 32 indices.  From 16 indices, or 32 columns, on the sliced product is the
+  // faster one at every size (16 indices: 6.2 us both; 128 rows, 128 indices, 1
+  // column: 10.3 against 22.6 us; 512 x 128 x 512, 512 nodes: 4.6 against 27.5 ms).
+  if (k <= 8 && n <= 16 && (long long)m * batch <= 16384) {
+    gemm_batched<double>(transA, transB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC,
+                         batch, st);
+    return;
+  }
+  const FxOperand a{A, lda, sA, transA}, b{B, ldb, sB, !transB};
+  fx_gemm(m, n, k, a, b, alpha, beta, C, ldc, sC, C, ldc, sC, batch, false, nullptr, 0, 0, st);
+}
+
+void dsyr2k_lower_batched(int m, int k, const double* A, int lda, long long sA, const double* P,
+                          int ldp, long long sP, const double* Q, int ldq, long long sQ, double* M,
+                          int ldm, long long sM, int batch, cudaStream_t st) {
+  if (m <= 0 || k <= 0 || batch <= 0) return;
+  // A - [P Q] [Q P]ᵀ
+  const FxOperand a{P, ldp, sP, false, Q, ldq, sQ}, b{Q, ldq, sQ, false, P, ldp, sP};
+  fx_gemm(m, m, 2 * k, a, b, -1.0, 1.0, A, lda, sA, M, ldm, sM, batch, true, nullptr, 0, 0, st);
+}
+
+void dsyrk_lower_batched(int m, int k, const double* A, int lda, long long sA, const double* P,
+                         int ldp, long long sP, double* M, int ldm, long long sM, double* PA,
+                         int ldpa, long long sPA, int batch, cudaStream_t st) {
+  if (m <= 0 || k <= 0 || batch <= 0) return;
+  const FxOperand a{P, ldp, sP, false};
+  fx_gemm(m, m, k, a, a, -1.0, 1.0, A, lda, sA, M, ldm, sM, batch, true, PA, ldpa, sPA, st);
+}

@@ -11,6 +11,7 @@
 
 #include "../../include/hss.h"
 #include "common.cuh"
+#include "fxgemm.cuh"
 
 namespace {
 
@@ -93,24 +94,24 @@ extern "C" int hss_matvec_noalloc(const hss_shape* shape, const double* D, const
       yh[l] = scratch + off + sz;
       off += 2 * sz;
     }
-    gemm_batched<double>(true, false, r, nc, leaf, 1.0, U, leaf, (long long)leaf * r, xc, ld, leaf,
+    dgemm_batched(true, false, r, nc, leaf, 1.0, U, leaf, (long long)leaf * r, xc, ld, leaf,
                          0.0, xh[L], nL * r, r, nL, st);
     for (int l = L - 1; l >= 1; --l)
-      gemm_batched<double>(true, false, r, nc, 2 * r, 1.0, E + eoff[l], 2 * r, 2 * rr, xh[l + 1],
+      dgemm_batched(true, false, r, nc, 2 * r, 1.0, E + eoff[l], 2 * r, 2 * rr, xh[l + 1],
                            (2 << l) * r, 2 * r, 0.0, xh[l], (1 << l) * r, r, 1 << l, st);
     for (int l = 1; l <= L; ++l) {
       const int ldl = (1 << l) * r;
-      gemm_batched<double>(false, false, r, nc, r, 1.0, S + soff[l], r, rr, xh[l], ldl, 2 * r, 0.0,
+      dgemm_batched(false, false, r, nc, r, 1.0, S + soff[l], r, rr, xh[l], ldl, 2 * r, 0.0,
                            yh[l] + r, ldl, 2 * r, 1 << (l - 1), st);
-      gemm_batched<double>(true, false, r, nc, r, 1.0, S + soff[l], r, rr, xh[l] + r, ldl, 2 * r,
+      dgemm_batched(true, false, r, nc, r, 1.0, S + soff[l], r, rr, xh[l] + r, ldl, 2 * r,
                            0.0, yh[l], ldl, 2 * r, 1 << (l - 1), st);
     }
     for (int l = 1; l <= L - 1; ++l)
-      gemm_batched<double>(false, false, 2 * r, nc, r, 1.0, E + eoff[l], 2 * r, 2 * rr, yh[l],
+      dgemm_batched(false, false, 2 * r, nc, r, 1.0, E + eoff[l], 2 * r, 2 * rr, yh[l],
                            (1 << l) * r, r, 1.0, yh[l + 1], (2 << l) * r, 2 * r, 1 << l, st);
-    gemm_batched<double>(false, false, leaf, nc, leaf, 1.0, D, leaf, (long long)leaf * leaf, xc, ld,
+    dgemm_batched(false, false, leaf, nc, leaf, 1.0, D, leaf, (long long)leaf * leaf, xc, ld,
                          leaf, 0.0, yc, ld, leaf, nL, st);
-    gemm_batched<double>(false, false, leaf, nc, r, 1.0, U, leaf, (long long)leaf * r, yh[L],
+    dgemm_batched(false, false, leaf, nc, r, 1.0, U, leaf, (long long)leaf * r, yh[L],
                          nL * r, r, 1.0, yc, ld, leaf, nL, st);
     if (cudaGetLastError() != cudaSuccess) return HSS_ERR_CUDA;
   }
