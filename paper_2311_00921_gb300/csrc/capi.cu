@@ -17,6 +17,7 @@
 
 #include "../../include/hss.h"
 #include "basis.cuh"
+#include "chol64.cuh"
 #include "common.cuh"
 #include "dfgemm.cuh"
 #include "fxgemm.cuh"
@@ -32,7 +33,7 @@ namespace {
 constexpr int kMaxCols = 32;      // right-hand-side columns per matvec pass
 constexpr int kSolveCols = 16;    // columns per triangular-sweep / refinement pass
 constexpr int kPanel = 32;        // columns per blocked-Cholesky panel (the panel kernel's limit)
-constexpr int kRootPanels = 16;
+constexpr int kTreeRank = 16;     // FP64 solves up to this rank run on the per-node kernels
 constexpr int kFuseNodes = 64;    // levels up to this many nodes apply Q inside the sweep kernel
 constexpr int kTreeTop = 6;       // levels 1 .. 6 (<= 64 nodes): one tree launch per direction
 
@@ -46,6 +47,8 @@ struct LevelT {
   T* A = nullptr;   // n x b x b merged blocks (levels < L), 1 block at the root
   T* B = nullptr;   // n x b x r bases fed to the QL (levels 1 .. L-1)
   T* yv = nullptr;  // level vector of the solve: (n b) x kSolveCols
+  T* Li = nullptr;  // FP64: inverted diagonal blocks of L^RR (chol64.cuh)
+  T* zv = nullptr;  // FP64: the forward sweep's z^R, laid out as yv
 };
 
 template <typename T>
@@ -53,6 +56,7 @@ struct Factor {
   std::vector<LevelT<T>> lv;   // index = level (0 = root)
   T *W = nullptr, *Y = nullptr, *X = nullptr, *Z = nullptr;
   T *t1 = nullptr, *t2 = nullptr;   // r x kSolveCols per node: Q application of wide levels
+  T* P = nullptr;                   // FP64: rows below a Cholesky block, n_L x leaf x 64
   const T *D = nullptr, *U = nullptr, *E = nullptr, *S = nullptr;   // generators in T
   T *Dc = nullptr, *Uc = nullptr, *Ec = nullptr, *Sc = nullptr;     // converted copies (float)
   T* d = nullptr;               // n x kSolveCols refinement correction (float)
@@ -92,13 +96,11 @@ struct hss_s {
   double* R0 = nullptr;                // FP64 root block of a mixed factor (2r x 2r)
   double* root_vec = nullptr;          // FP64 root vector of a mixed solve (2r x kSolveCols)
   double* root_vec2 = nullptr;
-  double* A0inv = nullptr;             // FP64 inverse of the root block (mixed solves)
-  int a0inv_valid = 0;
   double* rbuf = nullptr;              // n x kSolveCols residual
   double* bbuf = nullptr;              // n x kSolveCols copy of b (x aliasing b)
   double* norms = nullptr;             // 6 x kSolveCols: |b|, 1/|b|, |r|, 1/|r|, |x|, 1/|x|
   double* norm_part = nullptr;         // 64 x kSolveCols partial sums of the column norms
-  double* logdet_part = nullptr;       // 2^(L+1) - 1 node contributions
+  double* logdet_part = nullptr;       // 2^(L+1) - 1 node contributions, the root's first
   double* logdet_val = nullptr;
   int* status = nullptr;
   void* arena = nullptr;
@@ -192,7 +194,12 @@ void layout_factor(Bump& bp, Factor<T>& f, int L, int leaf, int r) {
     }
     if (l >= 1 && l < L) P.B = bp.take<T>((size_t)P.n * P.b * r);
     if (l < L) P.yv = bp.take<T>((size_t)P.n * P.b * kSolveCols);
+    if (sizeof(T) == 8) {
+      P.Li = bp.take<T>((size_t)P.n * inv_size(P.c));
+      P.zv = bp.take<T>((size_t)P.n * P.b * kSolveCols);
+    }
   }
+  if (sizeof(T) == 8) f.P = bp.take<T>(nL * std::max(leaf, 2) * 64);
   f.W = bp.take<T>(nL * leaf * r);
   f.Y = bp.take<T>(nL * leaf * r);
   f.X = bp.take<T>(nL * r * r);
@@ -239,14 +246,13 @@ size_t layout_main(hss_s* h, char* base) {
   }
   h->zq64 = bp.take<double>((size_t)nL * r * r);
   h->R0 = bp.take<double>((size_t)4 * r * r);
-  h->A0inv = bp.take<double>((size_t)4 * r * r);
   h->root_vec = bp.take<double>((size_t)2 * r * kSolveCols);
   h->root_vec2 = bp.take<double>((size_t)2 * r * kSolveCols);
   h->rbuf = bp.take<double>((size_t)h->n * kSolveCols);
   h->bbuf = bp.take<double>((size_t)h->n * kSolveCols);
   h->norms = bp.take<double>(6 * kSolveCols);
   h->norm_part = bp.take<double>(64 * kSolveCols);
-  h->logdet_part = bp.take<double>((size_t)(2 * nL - 1) + kRootPanels);
+  h->logdet_part = bp.take<double>((size_t)(2 * nL - 1));
   h->logdet_val = bp.take<double>(1);
   h->status = bp.take<int>(8);
   for (Lane& ln : h->lane) {
@@ -336,6 +342,17 @@ struct Launch {
   }
 };
 
+// the level routines' hook: runs fn, one launch, with the accounting of Launch
+struct LaunchLog {
+  hss_s* h;
+  cudaStream_t st;
+  template <typename F>
+  void operator()(int kind, double flops, F&& fn) const {
+    Launch k(h, kind, flops, st);
+    fn();
+  }
+};
+
 // Hooks of the basis completion chain: the same accounting as Launch, opened
 // before and closed after each of its launches.
 struct BasisTrace {
@@ -389,8 +406,7 @@ void gemm(hss_s* h, bool ta, bool tb, int m, int n, int k, T alpha, const T* A, 
     gemm_batched<T>(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, st);
 }
 
-// A - P Qᵀ - Q Pᵀ and A - P Pᵀ on the lower triangle, the latter with the merge
-// into the parents' blocks PA where given
+// A - P Qᵀ - Q Pᵀ on the lower triangle
 template <typename T>
 void syr2k(int m, int k, const T* A, int lda, long long sA, const T* P, int ldp, long long sP,
            const T* Q, int ldq, long long sQ, T* M, int ldm, long long sM, int batch,
@@ -399,17 +415,6 @@ void syr2k(int m, int k, const T* A, int lda, long long sA, const T* P, int ldp,
     dsyr2k_lower_batched(m, k, A, lda, sA, P, ldp, sP, Q, ldq, sQ, M, ldm, sM, batch, st);
   else
     syr2k_lower_batched<T>(m, k, A, lda, sA, P, ldp, sP, Q, ldq, sQ, M, ldm, sM, batch, st);
-}
-
-template <typename T>
-void syrk(int m, int k, const T* A, int lda, long long sA, const T* P, int ldp, long long sP, T* M,
-          int ldm, long long sM, T* PA, int ldpa, long long sPA, int batch, cudaStream_t st) {
-  if constexpr (std::is_same<T, double>::value)
-    dsyrk_lower_batched(m, k, A, lda, sA, P, ldp, sP, M, ldm, sM, PA, ldpa, sPA, batch, st);
-  else if (PA)
-    syrk_lower_merge_batched<T>(m, k, A, lda, sA, P, ldp, sP, M, ldm, sM, PA, ldpa, sPA, batch, st);
-  else
-    syrk_lower_batched<T>(m, k, A, lda, sA, P, ldp, sP, M, ldm, sM, batch, st);
 }
 
 // partial Cholesky of the first c of b columns: POTRF c x c, TRSM (b-c) x c,
@@ -537,26 +542,34 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
       Launch k(h, HSS_K_SYR2K, 2.0 * r * b * (b + 1.0) * n, st, sizeof(T) == 4);
       syr2k<T>(b, r, Ain, b, bb, f.Y, b, br, P.V, b, br, P.M, b, bb, n, st);
     }
-    // (c) partial Cholesky of the first c columns, blocked over the whole level:
-    // per panel of kPanel columns a per-node panel kernel (diagonal block and
-    // the rows below it) and one SYRK of every node's trailing lower triangle
+    // (c) partial Cholesky of the first c columns, blocked over the whole level
     double* slots = h->logdet_part + ((1LL << l) - 1);
     if (c == 0 && cudaMemsetAsync(slots, 0, sizeof(double) * n, st) != cudaSuccess)
       return HSS_ERR_CUDA;
-    for (int k0 = 0; k0 < c; k0 += kPanel) {
-      const int kb = std::min(kPanel, c - k0), rows = b - k0, nt = rows - kb;
-      T* Mk = P.M + k0 + (long long)k0 * b;
-      {
-        Launch k(h, HSS_K_PCHOL, panel_flops(rows, kb) * n, st, sizeof(T) == 4);
-        HSS_TRY(launch_chol_panel<T>(Mk, b, bb, rows, kb, slots, l, 0, k0, h->status, n, k0 > 0,
-                                     st));
-      }
-      if (nt > 0) {
-        Launch k(h, HSS_K_SYR2K, (double)nt * (nt + 1.0) * kb * n, st, sizeof(T) == 4);
-        T* Tr = Mk + kb + (long long)kb * b;
-        // the last update leaves Â^SS: its epilogue is the merge
-        syrk<T>(nt, kb, Tr, b, bb, Mk + kb, b, bb, Tr, b, bb, k0 + kb == c ? Q.A : nullptr, ldq,
-                sq, n, st);
+    if constexpr (std::is_same<T, double>::value) {
+      HSS_TRY(chol_level64({n, b, c, P.M, P.Li}, f.P, slots, l, 0, h->status, Q.A, ldq, sq, st,
+                           LaunchLog{h, st}));
+    } else {
+      // FP32: per panel of kPanel columns a per-node panel kernel (diagonal block
+      // and the rows below it) and one SYRK of every node's trailing lower triangle
+      for (int k0 = 0; k0 < c; k0 += kPanel) {
+        const int kb = std::min(kPanel, c - k0), rows = b - k0, nt = rows - kb;
+        T* Mk = P.M + k0 + (long long)k0 * b;
+        {
+          Launch k(h, HSS_K_PCHOL, panel_flops(rows, kb) * n, st, true);
+          HSS_TRY(launch_chol_panel<T>(Mk, b, bb, rows, kb, slots, l, 0, k0, h->status, n, k0 > 0,
+                                       st));
+        }
+        if (nt > 0) {
+          Launch k(h, HSS_K_SYR2K, (double)nt * (nt + 1.0) * kb * n, st, true);
+          T* Tr = Mk + kb + (long long)kb * b;
+          // the last update leaves Â^SS: its epilogue is the merge
+          if (k0 + kb == c)
+            syrk_lower_merge_batched<T>(nt, kb, Tr, b, bb, Mk + kb, b, bb, Tr, b, bb, Q.A, ldq, sq,
+                                        n, st);
+          else
+            syrk_lower_batched<T>(nt, kb, Tr, b, bb, Mk + kb, b, bb, Tr, b, bb, n, st);
+        }
       }
     }
     // (d, second half) with nothing eliminated (c = 0) Â^SS is the whole block:
@@ -571,39 +584,9 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
   return HSS_OK;
 }
 
-// Blocked right-looking Cholesky of the FP64 root block (last step of Alg. 2):
-// per 32-column panel, the diagonal block and the rows below it with the rows
-// split over CTAs of 32 rows, then the trailing update as a batch of 16-column
-// blocks, so that neither step queues on one SM's FP64 pipe.
-int root_cholesky(hss_s* h, double* R, int b0, cudaStream_t st) {
-  double* slots = h->logdet_part + ((2LL << h->L) - 1);
-  if (cudaMemsetAsync(slots, 0, kRootPanels * sizeof(double), st) != cudaSuccess ||
-      cudaMemsetAsync(h->logdet_part, 0, sizeof(double), st) != cudaSuccess)
-    return HSS_ERR_CUDA;
-  for (int k0 = 0, p = 0; k0 < b0; k0 += kPanel, ++p) {
-    const int kb = std::min(kPanel, b0 - k0), rows = b0 - k0;
-    double* Mk = R + k0 + (long long)k0 * b0;
-    {
-      Launch k(h, HSS_K_PCHOL, panel_flops(rows, kb), st);
-      HSS_TRY(launch_chol_panel<double>(Mk, b0, 0, rows, kb, slots + p, 0, 0, k0, h->status, 1,
-                                        false, st, std::max(1, (rows - kb + 31) / 32)));
-    }
-    const int nt = rows - kb;
-    if (nt > 0) {
-      double* P = Mk + kb;   // rows below the panel
-      double* C = R + (k0 + kb) + (long long)(k0 + kb) * b0;
-      // column block j (16 columns) of the trailing matrix: C_j -= P P_jᵀ, all
-      // blocks in one batched launch; a last partial block on its own
-      const int nb16 = nt / 16, tail = nt - 16 * nb16;
-      if (nb16 > 0)
-        gemm<double>(h, false, true, nt, 16, kb, -1.0, P, b0, 0, P, b0, 16, 1.0, C, b0,
-                     16LL * b0, nb16, st);
-      if (tail > 0)
-        gemm<double>(h, false, true, nt, tail, kb, -1.0, P, b0, 0, P + 16 * nb16, b0, 0, 1.0,
-                     C + 16LL * nb16 * b0, b0, 0, 1, st);
-    }
-  }
-  return check_launch();
+// the FP64 root block R as a level of one node with every column eliminated
+Level64 root_level(hss_s* h, double* R) {
+  return {1, 2 * h->rank, 2 * h->rank, R, h->f64.lv[0].Li};
 }
 
 int factorize(hss_s* h, int prec, cudaStream_t st) {
@@ -633,35 +616,11 @@ int factorize(hss_s* h, int prec, cudaStream_t st) {
     root = h->R0;
   }
   // root Cholesky (last step of Alg. 2), FP64 in every mode
-  const int b0 = 2 * r;
-  int rc = root_cholesky(h, root, b0, st);
-  if (rc) return rc;
+  HSS_TRY(chol_level64(root_level(h, root), h->f64.P, h->logdet_part, 0, 0, h->status, nullptr, 0,
+                       0, st, LaunchLog{h, st}));
   {
     Launch k(h, HSS_K_OTHER, (double)((2LL << L) - 1), st);
-    launch_logdet_reduce(h->logdet_part, (int)((2LL << L) - 1) + kRootPanels, h->logdet_val, st);
-  }
-  // mixed modes: the root solve of every refinement pass multiplies by the FP64
-  // inverse of the root block, formed here from its Cholesky factor with the
-  // triangular sweeps run on the identity, 16 columns per CTA
-  h->a0inv_valid = 0;
-  if (prec != HSS_FP64 && b0 % kSolveCols == 0) {
-    {
-      Launch k(h, HSS_K_OTHER, 0.0, st);
-      launch_eye(h->A0inv, b0, st);
-    }
-    const int chunks = b0 / kSolveCols;
-    const long long sx = (long long)kSolveCols * b0;
-    {
-      Launch k(h, HSS_K_TRSV_FWD, trsv_flops(b0, b0, b0), st);
-      HSS_TRY(launch_trsv_fwd<double>(root, b0, 0, b0, b0, h->A0inv, b0, sx, kSolveCols, nullptr,
-                                      0, 0, chunks, st));
-    }
-    {
-      Launch k(h, HSS_K_TRSV_BWD, trsv_flops(b0, b0, b0), st);
-      HSS_TRY(launch_trsv_bwd<double>(root, b0, 0, b0, b0, h->A0inv, b0, sx, kSolveCols, nullptr,
-                                      0, 0, chunks, st));
-    }
-    h->a0inv_valid = 1;
+    launch_logdet_reduce(h->logdet_part, (int)((2LL << L) - 1), h->logdet_val, st);
   }
   return check_launch();
 }
@@ -685,6 +644,48 @@ void apply_q(hss_s* h, Factor<T>& f, const LevelT<T>& P, T* vec, int ldv, int nc
           b, n, st);
 }
 
+// root solve on nc columns of y (2 rank rows), z: scratch of the same size
+int solve_root(hss_s* h, double* R, double* y, double* z, int nc, cudaStream_t st) {
+  const int b0 = 2 * h->rank;
+  const Level64 lv = root_level(h, R);
+  HSS_TRY(fwd_level64(lv, y, b0, z, b0, nullptr, 0, nc, st, LaunchLog{h, st}));
+  HSS_TRY(bwd_level64(lv, y, b0, z, b0, nullptr, 0, nc, st, LaunchLog{h, st}));
+  return HSS_OK;
+}
+
+// The FP64 ULV sweeps as products over whole levels: Q by three, each triangular
+// sweep by two per 128 eliminated columns (chol64.cuh).  A node's sweep in one CTA
+// is bound by that SM's FP64 pipe, 540 us a level and direction at rank 128 with 16
+// columns (78 us at rank 32 with one) against 65 us (33 us) for the products; up
+// to rank kTreeRank the per-node kernels, one launch for all upper levels, are as
+// fast or faster and stay.
+int solve_levels64(hss_s* h, double* x, int nc, int ld, cudaStream_t st) {
+  const int L = h->L;
+  Factor<double>& f = h->f64;
+  const LaunchLog log{h, st};
+  auto level = [&](int l) {
+    const LevelT<double>& P = f.lv[l];
+    return Level64{P.n, P.b, P.c, P.M, P.Li};
+  };
+  for (int l = L; l >= 1; --l) {
+    const LevelT<double>&P = f.lv[l], &Q = f.lv[l - 1];
+    double* vec = l == L ? x : P.yv;
+    const int ldz = P.n * P.b, ldv = l == L ? ld : ldz;
+    apply_q<double>(h, f, P, vec, ldv, nc, /*transpose=*/true, st, 0);
+    HSS_TRY(fwd_level64(level(l), vec, ldv, P.zv, ldz, Q.yv, Q.n * Q.b, nc, st, log));
+  }
+  const int rc = solve_root(h, f.lv[0].A, f.lv[0].yv, f.lv[0].zv, nc, st);
+  if (rc) return rc;
+  for (int l = 1; l <= L; ++l) {
+    const LevelT<double>&P = f.lv[l], &Q = f.lv[l - 1];
+    double* vec = l == L ? x : P.yv;
+    const int ldz = P.n * P.b, ldv = l == L ? ld : ldz;
+    HSS_TRY(bwd_level64(level(l), vec, ldv, P.zv, ldz, Q.yv, Q.n * Q.b, nc, st, log));
+    apply_q<double>(h, f, P, vec, ldv, nc, /*transpose=*/false, st, 0);
+  }
+  return check_launch();
+}
+
 // The ULV sweeps on nc <= kSolveCols columns of x (in place), arithmetic T;
 // the root solve is FP64 in every mode.  Lane g uses columns col0 .. col0+nc-1
 // of every level vector and scratch block, and its own tree flags.
@@ -692,6 +693,9 @@ template <typename T>
 int solve_sweeps(hss_s* h, Factor<T>& f, T* x, int nc, int ld, cudaStream_t st, int g = 0,
                  int col0 = 0) {
   const int L = h->L, r = h->rank;
+  if constexpr (std::is_same<T, double>::value) {
+    if (r > kTreeRank) return solve_levels64(h, x, nc, ld, st);
+  }
   Lane& ln = h->lane[g];
   // level l's vector, this lane's columns
   auto lvec = [&](int l) { return f.lv[l].yv + (long long)col0 * f.lv[l].n * f.lv[l].b; };
@@ -744,20 +748,10 @@ int solve_sweeps(hss_s* h, Factor<T>& f, T* x, int nc, int ld, cudaStream_t st, 
     Launch k(h, HSS_K_OTHER, 0.0, st);
     launch_f32_to_f64(reinterpret_cast<const float*>(lvec(0)), rv, (long long)b0 * nc, st);
   }
-  if (sizeof(T) != sizeof(double) && h->a0inv_valid) {
-    gemm<double>(h, false, false, b0, nc, b0, 1.0, h->A0inv, b0, 0, rv, b0, 0, 0.0,
-                 h->root_vec2 + rc0, b0, 0, 1, st);
-    rv = h->root_vec2 + rc0;
-  } else {
-    {
-      Launch k(h, HSS_K_TRSV_FWD, trsv_flops(b0, b0, nc), st);
-      HSS_TRY(launch_trsv_fwd<double>(rootA, b0, 0, b0, b0, rv, b0, 0, nc, nullptr, 0, 0, 1, st));
-    }
-    {
-      Launch k(h, HSS_K_TRSV_BWD, trsv_flops(b0, b0, nc), st);
-      HSS_TRY(launch_trsv_bwd<double>(rootA, b0, 0, b0, b0, rv, b0, 0, nc, nullptr, 0, 0, 1, st));
-    }
-  }
+  int rc = solve_root(h, rootA, rv, sizeof(T) == sizeof(double)
+                                        ? reinterpret_cast<double*>(f.lv[0].zv)
+                                        : h->root_vec2 + rc0, nc, st);
+  if (rc) return rc;
   if (sizeof(T) != sizeof(double)) {
     Launch k(h, HSS_K_OTHER, 0.0, st);
     launch_f64_to_f32(rv, reinterpret_cast<float*>(lvec(0)), (long long)b0 * nc, st);

@@ -33,7 +33,7 @@
 
 #include <map>
 #include <mutex>
-#include <tuple>
+#include <utility>
 
 #include "common.cuh"
 #include "fxgemm.cuh"
@@ -385,23 +385,6 @@ fx_gemm_kernel(const __grid_constant__ FxShape s) {
     }
 }
 
-// dynamic shared memory above the default, once per device and kernel
-template <typename F>
-cudaError_t allow_smem(F kernel, int bytes) {
-  static std::mutex mu;
-  static std::map<std::tuple<int, const void*>, cudaError_t> memo;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const auto key = std::make_tuple(dev, reinterpret_cast<const void*>(kernel));
-  std::lock_guard<std::mutex> g(mu);
-  const auto it = memo.find(key);
-  if (it != memo.end()) return it->second;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  memo[key] = e;
-  return e;
-}
-
 template <int BN, bool AKC, bool BKC>
 cudaError_t launch(FxShape& s, int batch, cudaStream_t st) {
   s.tiles_m = (s.m + kRows - 1) / kRows;
@@ -414,7 +397,8 @@ cudaError_t launch(FxShape& s, int batch, cudaStream_t st) {
       s.tiles += have < s.tiles_n ? have : s.tiles_n;
     }
   }
-  const cudaError_t e = allow_smem(fx_gemm_kernel<BN, AKC, BKC>, fx_smem<BN>());
+  const cudaError_t e = fx_allow_smem(
+      reinterpret_cast<const void*>(fx_gemm_kernel<BN, AKC, BKC>), fx_smem<BN>());
   if (e != cudaSuccess) return e;
   fx_gemm_kernel<BN, AKC, BKC>
       <<<(unsigned)((long long)s.tiles * batch), kThreads, fx_smem<BN>(), st>>>(s);
@@ -428,6 +412,21 @@ cudaError_t launch_modes(FxShape& s, int batch, cudaStream_t st) {
 }
 
 }  // namespace
+
+cudaError_t fx_allow_smem(const void* kernel, int bytes) {
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, cudaError_t> memo;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> g(mu);
+  const auto key = std::make_pair(dev, kernel);
+  const auto it = memo.find(key);
+  if (it != memo.end()) return it->second;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  memo[key] = e;
+  return e;
+}
 
 cudaError_t fx_gemm(int m, int n, int K, const FxOperand& a, const FxOperand& b, double alpha,
                     double beta, const double* Cin, int ldcin, long long sCin, double* C, int ldc,

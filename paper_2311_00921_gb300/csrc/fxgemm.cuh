@@ -24,6 +24,9 @@ cudaError_t fx_gemm(int m, int n, int K, const FxOperand& a, const FxOperand& b,
                     long long sC, int batch, bool lower, double* PA, int ldpa, long long sPA,
                     cudaStream_t st);
 
+// opts a kernel into `bytes` of dynamic shared memory, once per device and kernel
+cudaError_t fx_allow_smem(const void* kernel, int bytes);
+
 // The FP64 products of the library, column-major with batch strides in elements
 // (semantics of gemm_batched, syr2k_lower_batched, syrk_lower_batched and
 // syrk_lower_merge_batched in common.cuh): sliced products except where the rule

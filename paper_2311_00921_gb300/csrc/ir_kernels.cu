@@ -82,12 +82,6 @@ __global__ void col_norms_final_kernel(const double* __restrict__ part, int nc, 
   }
 }
 
-__global__ void eye_kernel(double* a, int n) {
-  for (long long e = blockIdx.x * (long long)NT + threadIdx.x; e < (long long)n * n;
-       e += (long long)gridDim.x * NT)
-    a[e] = (e % n == e / n) ? 1.0 : 0.0;
-}
-
 int grid_for(long long n) {
   long long g = (n + NT - 1) / NT;
   return (int)(g < 152 * 16 ? (g < 1 ? 1 : g) : 152 * 16);
@@ -127,9 +121,6 @@ void launch_col_norms(const double* v, int ld, int m, int nc, double* norms, dou
   col_norms_final_kernel<<<(nc + 7) / 8, 256, 0, st>>>(scratch, nc, norms, inv);
 }
 
-void launch_eye(double* a, int n, cudaStream_t st) {
-  eye_kernel<<<grid_for((long long)n * n), NT, 0, st>>>(a, n);
-}
 
 __global__ void fill_test_kernel(double* x, int n, int nc) {
   const int j = blockIdx.y;

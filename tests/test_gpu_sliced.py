@@ -77,3 +77,40 @@ def test_values_outside_the_sliced_range():
     for j in (0, 3, 5, 7, 8, 9, 11):
         ref = np.einsum("zij,zj->zi", D.astype(LD), x[:, :, j].astype(LD))
         assert np.all(np.abs(y[:, :, j] - ref) <= (leaf + 4) * 2.0 ** -53 * np.abs(ref)), j
+
+
+@pytest.mark.parametrize("leaf,rank,nrhs", [
+    (18, 17, 1), (49, 17, 3), (81, 17, 16), (82, 17, 17), (145, 17, 2), (146, 18, 9),
+    (300, 40, 5), (256, 130, 1), (20, 20, 4)])
+def test_blocked_levels_against_oracle(leaf, rank, nrhs):
+    """The FP64 level routines at the edges of their blocks (1, 32, 64, 128 and more
+    eliminated columns, ragged ones, none), with the tolerances of the parity tests."""
+    from oracle import ulv as O
+    from paper_2311_00921_gb300 import inputs as I
+    h = I.random_hss(3, leaf, rank, seed=leaf + rank, orthonormal=False)
+    F, b = O.factor(h), I.rhs(h.n, nrhs, 7)
+    x_ref, ld_ref = O.solve(F, b), O.logdet(F)
+    dev = hss.HSS(h)
+    dev.factorize("fp64")
+    x = dev.solve(hss.colmajor(b)).cpu().numpy()
+    err = np.linalg.norm(x - x_ref, axis=0) / np.linalg.norm(x_ref, axis=0)
+    assert err.max() <= 1e-10
+    assert abs(dev.logdet() - ld_ref) <= 1e-12 * abs(ld_ref)
+
+
+def test_pivot_in_a_later_block():
+    """A block whose first non-positive pivot lies past the first 64 columns is
+    reported at the oracle's column."""
+    from oracle import ulv as O
+    from paper_2311_00921_gb300 import inputs as I
+    h = I.random_hss(2, 200, 20, seed=9)
+    h.D[2][:100, :100] -= 2.0 * np.diag(np.diag(h.D[2])[:100])
+    dev = hss.HSS(h)
+    dev.factorize("fp64")
+    assert dev.last_info()["code"] == -3
+    with pytest.raises(O.NotSPD) as eo:
+        O.factor(h)
+    info = dev.last_info()
+    assert (info["level"], info["node"], info["col"]) == (eo.value.level, eo.value.node,
+                                                         eo.value.col)
+    assert info["col"] > 64
