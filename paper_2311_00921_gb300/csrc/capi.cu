@@ -22,6 +22,7 @@
 #include "dfgemm.cuh"
 #include "fxgemm.cuh"
 #include "ir_kernels.cuh"
+#include "qlpanel.cuh"
 #include "tc_gemm.cuh"
 #include "ulv_kernels.cuh"
 #include "uneven.cuh"
@@ -346,9 +347,10 @@ struct Launch {
 struct LaunchLog {
   hss_s* h;
   cudaStream_t st;
+  bool f32 = false;
   template <typename F>
   void operator()(int kind, double flops, F&& fn) const {
-    Launch k(h, kind, flops, st);
+    Launch k(h, kind, flops, st, f32);
     fn();
   }
 };
@@ -433,6 +435,17 @@ double qapply_flops(int b, int r, int nrhs) { return (4.0 * b * r + 2.0 * r * r)
 enum { SPLIT_D = 1, SPLIT_U = 2, SPLIT_E = 4, SPLIT_S = 8, SPLIT_ALL = 15 };
 cudaError_t split_generators(hss_s* h, cudaStream_t st, int which, bool lo);
 
+// Whether the Householder basis completion runs as panels and level-wide products.
+// In FP64 from the second 16-column panel on (level of 256 x 128 bases, any node
+// count up to the SMs: 2.7 -> 1.45 ms; 512 leaves of 512 x 128: 18.9 -> 8.4 ms; 16 of
+// 256 x 32: 0.29 -> 0.24 ms).  In FP32 the one-CTA kernel's products are fast and the
+// launches count: rank 96 loses 2 % of a step, rank 256 gains (leaf 1024: 8.9 ->
+// 3.1 ms, the levels above 2.2 -> 1.3 ms).
+template <typename T>
+bool ql_blocked(int r) {
+  return r > (sizeof(T) == 8 ? 16 : 128);
+}
+
 // levels L .. 1 of Alg. 2; leaves the merged root block in f.lv[0].A.
 // Two chains: the basis chain (basis completion of level l, then the merge's
 // rescaled coupling Ŝ and the parent basis, which need only L_B of level l) runs
@@ -471,6 +484,10 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
       hook.ctx = &bt;
       HSS_TRY(launch_basis_completion<T>(Bsrc, br, P.V, br, P.T_, rr, P.LB, rr, b, r, n, f.bs,
                                          hook, qs));
+    } else if (ql_blocked<T>(r)) {
+      if (sizeof(T) == 8 && !ql_accepts64(b, r)) return HSS_ERR_INVALID_ARG;
+      HSS_TRY(ql_level<T>(Bsrc, P.V, P.T_, P.LB, b, r, n, f.bs.X, f.bs.G, f.bs.R1, h->ql_panel, qs,
+                          LaunchLog{h, qs, sizeof(T) == 4}));
     } else {
       Launch k(h, HSS_K_QL, (2.0 * b * r * r - 2.0 / 3.0 * r * r * r + 1.0 * b * r * r) * n, qs,
                sizeof(T) == 4);
@@ -527,6 +544,9 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
     }
     if (!tc)
       gemm<T>(h, false, false, b, r, b, T(1), Ain, b, bb, P.V, b, br, T(0), f.W, b, br, n, st);
+    if (ql_blocked<T>(r) && !(h->basis_method == HSS_BASIS_CHOLQR && r <= basis_max_rank<T>()))
+      HSS_TRY(ql_tfactor<T>(P.V, P.T_, b, r, n, f.bs.R, f.bs.P, st,
+                            LaunchLog{h, st, sizeof(T) == 4}));
     gemm<T>(h, false, false, b, r, r, T(1), f.W, b, br, P.T_, r, rr, T(0), f.Y, b, br, n, st);
     gemm<T>(h, true, false, r, r, b, T(1), P.V, b, br, f.Y, b, br, T(0), f.X, r, rr, n, st);
     gemm<T>(h, true, false, r, r, r, T(1), P.T_, r, rr, f.X, r, rr, T(0), f.Z, r, rr, n, st);

@@ -18,21 +18,6 @@ constexpr int kT = 128;   // threads
 constexpr int kN = 64;    // order of the block
 constexpr int kP = 65;    // pitch of its columns in shared memory
 
-// 1 / sqrt(d), d > 0: y0 from FP32 on d scaled to [1, 4) by a power of four, then
-// y = y0 + y0 e (1/2 + 3/8 e), e = 1 - d y0² (Newton's iteration with the second
-// term of the series kept): the estimate's 2^-22 becomes 2^-63 before rounding.
-HSS_DEVINL double inv_sqrt(double d) {
-  const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
-  if (ex == 0 || ex == 0x7ff) return 1.0 / sqrt(d);
-  const int e = ex - 1023, p = e >> 1;
-  const double m =
-      __hiloint2double((hi & 0xfffff) | ((1023 + e - 2 * p) << 20), __double2loint(d));
-  const double y0 = (double)rsqrtf((float)m);
-  const double r = fma(-m, y0 * y0, 1.0);
-  const double y = fma(y0 * r, fma(0.375, r, 0.5), y0);
-  return __hiloint2double(__double2hiint(y) - (p << 20), __double2loint(y));
-}
-
 // factor and inverse of the 32 x 32 diagonal block at offset o: S (L, lower) and X
 HSS_DEVINL void factor32(double* S, double* X, int o, double (*col)[32], double (*xrow)[32],
                          int level, int node, int col0, int* status) {

@@ -22,6 +22,33 @@ HSS_DEVINL void report_failure(int* status, int code, int level, int node, int c
   }
 }
 
+// 1 / sqrt(d), d > 0: y0 from FP32 on d scaled to [1, 4) by a power of four, then
+// y = y0 + y0 e (1/2 + 3/8 e), e = 1 - d y0² (Newton's iteration with the second
+// term of the series kept): the estimate's 2^-22 becomes 2^-63 before rounding.
+HSS_DEVINL double inv_sqrt(double d) {
+  const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
+  if (ex == 0 || ex == 0x7ff) return 1.0 / sqrt(d);
+  const int e = ex - 1023, p = e >> 1;
+  const double m =
+      __hiloint2double((hi & 0xfffff) | ((1023 + e - 2 * p) << 20), __double2loint(d));
+  const double y0 = (double)rsqrtf((float)m);
+  const double r = fma(-m, y0 * y0, 1.0);
+  const double y = fma(y0 * r, fma(0.375, r, 0.5), y0);
+  return __hiloint2double(__double2hiint(y) - (p << 20), __double2loint(y));
+}
+
+// 1 / d, d > 0, the same way: y = y0 (1 + e + e²), e = 1 - d y0, y0 the FP32 reciprocal
+// of d scaled to [1, 2)
+HSS_DEVINL double inv_pos(double d) {
+  const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
+  if (ex < 32 || ex > 0x7ff - 32) return 1.0 / d;
+  const double m = __hiloint2double((hi & 0xfffff) | (1023 << 20), __double2loint(d));
+  const double y0 = (double)(1.f / (float)m);
+  const double e = fma(-m, y0, 1.0);
+  const double y = fma(y0, fma(e, e, e), y0);
+  return __hiloint2double(__double2hiint(y) - ((ex - 1023) << 20), __double2loint(y));
+}
+
 template <typename T>
 HSS_DEVINL T warp_sum(T v) {
 #pragma unroll

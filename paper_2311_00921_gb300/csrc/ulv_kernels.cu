@@ -1346,6 +1346,10 @@ cudaError_t launch_ql_rows(const T* Bsrc, int ldb_src, long long sB, T* V, long 
   return cudaGetLastError();
 }
 
+bool ql_accepts64(int b, int r) {
+  return b <= 3 * NT || smem_opt_in(ql_basis_kernel<double, 16, 4>, ql_smem<double>(b, r, 16));
+}
+
 template <typename T>
 cudaError_t launch_ql_basis(const T* Bsrc, int ldb_src, long long sB, T* V, long long sV, T* Tm,
                             long long sT, T* LB, long long sL, int b, int r, int nodes,

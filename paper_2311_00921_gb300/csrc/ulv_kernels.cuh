@@ -11,6 +11,11 @@ cudaError_t launch_ql_basis(const T* Bsrc, int ldb_src, long long sB, T* V, long
                             long long sT, T* LB, long long sL, int b, int r, int nodes,
                             cudaStream_t st, const int* only_if = nullptr, int panel = 0);
 
+// Whether the FP64 factorization takes nodes of order b and rank r: those of the
+// one-CTA kernel's shared memory (every rank up to order 768, 176 at 1024).  The
+// blocked completion has no such limit but keeps to the documented one.
+bool ql_accepts64(int b, int r);
+
 template <typename T>
 size_t pchol_smem(int b);
 
