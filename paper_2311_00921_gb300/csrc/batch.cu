@@ -21,8 +21,10 @@
 #include <vector>
 
 #include "../../include/hss.h"
+#include "chol64.cuh"
 #include "common.cuh"
 #include "fxgemm.cuh"
+#include "qlpanel.cuh"
 #include "ulv_kernels.cuh"
 #include "uneven.cuh"
 
@@ -37,6 +39,9 @@ struct Height {
   int b = 0, c = 0;
   double *V = nullptr, *T = nullptr, *LB = nullptr, *M = nullptr, *A = nullptr, *B = nullptr;
   double *E = nullptr, *S = nullptr, *yv = nullptr, *ldp = nullptr;
+  double *Li = nullptr, *zv = nullptr;   // inverted diagonal blocks, forward sweep's z (chol64.cuh)
+
+  Level64 level() const { return {(int)nodes, b, c, M, Li}; }
 };
 
 struct Group {
@@ -48,6 +53,9 @@ struct Group {
   double *R = nullptr, *rootvec = nullptr, *ldroot = nullptr;
   double *W = nullptr, *Y = nullptr, *X = nullptr, *Z = nullptr, *Zq = nullptr;
   double *t1 = nullptr, *t2 = nullptr, *xg = nullptr;
+  double *qW = nullptr, *q1 = nullptr, *q2 = nullptr;   // basis chain's scratch (qlpanel.cuh)
+  double *tG = nullptr, *tP = nullptr, *cP = nullptr;   // main chain's: T factor, Cholesky rows
+  double *rootLi = nullptr, *rootz = nullptr;
   long long rows = 0;          // leaf-level rows of the group
   std::vector<long long> row_off;   // member -> row offset in xg
   cudaStream_t st = nullptr, qs = nullptr;
@@ -131,6 +139,8 @@ size_t layout(hss_batch_s* bt, char* base) {
         t.yv = bp.take<double>(t.nodes * t.b * kCols);
       }
       t.S = bp.take<double>((t.nodes / 2) * rr);
+      t.Li = bp.take<double>(t.nodes * inv_size(t.c));
+      t.zv = bp.take<double>(t.nodes * t.b * kCols);
       ldp_total += t.nodes;
     }
     const long long n0 = g.ht[0].nodes;
@@ -139,11 +149,16 @@ size_t layout(hss_batch_s* bt, char* base) {
     g.U = bp.take<double>(n0 * leaf * r);
     g.R = bp.take<double>((size_t)nm * 4 * rr);
     g.rootvec = bp.take<double>((size_t)nm * 2 * r * kCols);
+    g.rootz = bp.take<double>((size_t)nm * 2 * r * kCols);
+    g.rootLi = bp.take<double>((size_t)nm * inv_size(2 * r));
     g.W = bp.take<double>(n0 * leaf * r);
     g.Y = bp.take<double>(n0 * leaf * r);
     g.X = bp.take<double>(n0 * rr);
     g.Z = bp.take<double>(n0 * rr);
     g.Zq = bp.take<double>(n0 * rr);
+    g.qW = bp.take<double>(n0 * leaf * r);
+    for (double** p : {&g.q1, &g.q2, &g.tG, &g.tP}) *p = bp.take<double>(n0 * rr);
+    g.cP = bp.take<double>(n0 * std::max(leaf, 2) * 64);
     g.t1 = bp.take<double>(n0 * r * kCols);
     g.t2 = bp.take<double>(n0 * r * kCols);
     g.xg = bp.take<double>(g.rows * kCols);
@@ -189,6 +204,23 @@ void gemm(bool ta, bool tb, int m, int n, int k, double alpha, const double* A, 
       return e_ == cudaErrorInvalidConfiguration ? HSS_ERR_INVALID_ARG : HSS_ERR_CUDA; \
   } while (0)
 
+// the level routines' hook: no accounting here
+struct NoLog {
+  template <typename F>
+  void operator()(int, double, F&& fn) const {
+    fn();
+  }
+};
+
+Level64 root_level(const Group& g) {
+  return {(int)g.member.size(), 2 * g.r, 2 * g.r, g.R, g.rootLi};
+}
+
+// Basis completion, Cholesky and sweeps run as in the single path (qlpanel.cuh,
+// chol64.cuh): panels and products over a whole height of the group.  With a node
+// per CTA on that SM's FP64 pipe, a height cost 0.5 to 2 ms in the Cholesky and
+// 0.3 to 2.7 ms in the QL whatever its node count, and a group's heights follow
+// one another: 10 matrices of order 2,048 to 16,384 took 28.5 ms, now 12.7 ms.
 int factor_group(hss_batch_s* bt, Group& g) {
   const int r = g.r;
   const long long rr = (long long)r * r;
@@ -201,7 +233,12 @@ int factor_group(hss_batch_s* bt, Group& g) {
     const int b = t.b;
     const long long br = (long long)b * r;
     const double* Bsrc = (h == 0) ? g.U : t.B;
-    TRY(launch_ql_basis<double>(Bsrc, b, br, t.V, br, t.T, rr, t.LB, rr, b, r, (int)t.nodes, qs));
+    if (ql_blocked<double>(r))
+      TRY(ql_level<double>(Bsrc, t.V, t.T, t.LB, b, r, (int)t.nodes, g.qW, g.q1, g.q2, 0, qs,
+                           NoLog()));
+    else
+      TRY(launch_ql_basis<double>(Bsrc, b, br, t.V, br, t.T, rr, t.LB, rr, b, r, (int)t.nodes,
+                                  qs));
     const long long np = t.split / 2, nq = (t.nodes - t.split) / 2;
     // pairs with a regular parent at h + 1
     if (np > 0) {
@@ -238,24 +275,27 @@ int factor_group(hss_batch_s* bt, Group& g) {
     TRY(cudaStreamWaitEvent(st, g.ev[h], 0));
     const double* Ain = (h == 0) ? g.D : t.A;
     gemm(false, false, b, r, b, 1.0, Ain, b, bb, t.V, b, br, 0.0, g.W, b, br, n, st);
+    if (ql_blocked<double>(r))
+      TRY(ql_tfactor<double>(t.V, t.T, b, r, (int)n, g.tG, g.tP, st, NoLog()));
     gemm(false, false, b, r, r, 1.0, g.W, b, br, t.T, r, rr, 0.0, g.Y, b, br, n, st);
     gemm(true, false, r, r, b, 1.0, t.V, b, br, g.Y, b, br, 0.0, g.X, r, rr, n, st);
     gemm(true, false, r, r, r, 1.0, t.T, r, rr, g.X, r, rr, 0.0, g.Z, r, rr, n, st);
     gemm(false, false, b, r, r, -0.5, t.V, b, br, g.Z, r, rr, 1.0, g.Y, b, br, n, st);
     dsyr2k_lower_batched(b, r, Ain, b, bb, g.Y, b, br, t.V, b, br, t.M, b, bb, (int)n, st);
-    if (t.split > 0)
-      TRY(launch_pchol<double>(t.M, b, bb, b, c, g.ht[h + 1].A, 2 * r, 4 * rr, t.ldp, h, 0,
-                               bt->status, (int)t.split, st));
-    if (t.nodes > t.split)
-      TRY(launch_pchol<double>(t.M + t.split * bb, b, bb, b, c, g.R + (long long)t.mfirst * 4 * rr,
-                               2 * r, 4 * rr, t.ldp, h, (int)t.split, bt->status,
-                               (int)(t.nodes - t.split), st));
+    const Merge64 up{t.split > 0 ? g.ht[h + 1].A : nullptr, 2 * r, 4 * rr, (int)t.split,
+                     g.R + (long long)t.mfirst * 4 * rr};
+    if (c > 0) {
+      TRY(chol_level64(t.level(), g.cP, t.ldp, h, 0, bt->status, up, st, NoLog()));
+    } else {   // nothing eliminated: the blocks themselves go to the parents
+      TRY(cudaMemsetAsync(t.ldp, 0, sizeof(double) * n, st));
+      TRY(launch_scatter_ss<double>(t.M, b, bb, c, r, up.PA, up.ld, up.stride, up.split, st));
+      TRY(launch_scatter_ss<double>(t.M + t.split * bb, b, bb, c, r, up.PA2, up.ld, up.stride,
+                                    (int)(n - t.split), st));
+    }
     TRY(cudaGetLastError());
   }
-  // every member's root Cholesky in one launch
-  const int nm = (int)g.member.size();
-  TRY(launch_pchol<double>(g.R, 2 * r, 4 * rr, 2 * r, 2 * r, nullptr, 0, 0, g.ldroot, g.H, 0,
-                           bt->status, nm, st));
+  // every member's root Cholesky as one level
+  TRY(chol_level64(root_level(g), g.cP, g.ldroot, g.H, 0, bt->status, {}, st, NoLog()));
   return HSS_OK;
 }
 
@@ -275,42 +315,36 @@ int solve_group(Group& g, int nc) {
   const int r = g.r, nm = (int)g.member.size();
   cudaStream_t st = g.st;
   const int ldroot = nm * 2 * r;
-  for (int h = 0; h < g.H; ++h) {
+  const NoLog log;
+  // the parents' vectors of height h's nodes: those of h + 1 for the first `split`,
+  // root vectors for the others
+  auto sweep = [&](int h, bool fwd) -> cudaError_t {
     Height& t = g.ht[h];
     double* vec = (h == 0) ? g.xg : t.yv;
-    const int ldv = (h == 0) ? (int)g.rows : (int)(t.nodes * t.b);
-    const long long bb = (long long)t.b * t.b;
-    apply_q(g, t, vec, ldv, nc, true, st);
-    if (t.split > 0) {
+    const int ldz = (int)(t.nodes * t.b), ldv = (h == 0) ? (int)g.rows : ldz;
+    const int split = (int)t.split, rest = (int)t.nodes - split;
+    auto part = [&](int first, int count, double* par, int ldpar) {
+      double *y = vec + (long long)first * t.b, *z = t.zv + (long long)first * t.b;
+      const Level64 lv = t.level().part(first, count);
+      return fwd ? fwd_level64(lv, y, ldv, z, ldz, par, ldpar, nc, st, log)
+                 : bwd_level64(lv, y, ldv, z, ldz, par, ldpar, nc, st, log);
+    };
+    if (fwd) apply_q(g, t, vec, ldv, nc, true, st);
+    cudaError_t e = cudaSuccess;
+    if (split > 0) {
       Height& u = g.ht[h + 1];
-      TRY(launch_trsv_fwd<double>(t.M, t.b, bb, t.b, t.c, vec, ldv, t.b, nc, u.yv,
-                                  (int)(u.nodes * u.b), r, (int)t.split, st));
+      e = part(0, split, u.yv, (int)(u.nodes * u.b));
     }
-    if (t.nodes > t.split)
-      TRY(launch_trsv_fwd<double>(t.M + t.split * bb, t.b, bb, t.b, t.c, vec + t.split * t.b, ldv,
-                                  t.b, nc, g.rootvec + (long long)t.mfirst * 2 * r, ldroot, r,
-                                  (int)(t.nodes - t.split), st));
-  }
-  TRY(launch_trsv_fwd<double>(g.R, 2 * r, 4LL * r * r, 2 * r, 2 * r, g.rootvec, ldroot, 2 * r, nc,
-                              nullptr, 0, 0, nm, st));
-  TRY(launch_trsv_bwd<double>(g.R, 2 * r, 4LL * r * r, 2 * r, 2 * r, g.rootvec, ldroot, 2 * r, nc,
-                              nullptr, 0, 0, nm, st));
-  for (int h = g.H - 1; h >= 0; --h) {
-    Height& t = g.ht[h];
-    double* vec = (h == 0) ? g.xg : t.yv;
-    const int ldv = (h == 0) ? (int)g.rows : (int)(t.nodes * t.b);
-    const long long bb = (long long)t.b * t.b;
-    if (t.split > 0) {
-      Height& u = g.ht[h + 1];
-      TRY(launch_trsv_bwd<double>(t.M, t.b, bb, t.b, t.c, vec, ldv, t.b, nc, u.yv,
-                                  (int)(u.nodes * u.b), r, (int)t.split, st));
-    }
-    if (t.nodes > t.split)
-      TRY(launch_trsv_bwd<double>(t.M + t.split * bb, t.b, bb, t.b, t.c, vec + t.split * t.b, ldv,
-                                  t.b, nc, g.rootvec + (long long)t.mfirst * 2 * r, ldroot, r,
-                                  (int)(t.nodes - t.split), st));
-    apply_q(g, t, vec, ldv, nc, false, st);
-  }
+    if (e == cudaSuccess && rest > 0)
+      e = part(split, rest, g.rootvec + (long long)t.mfirst * 2 * r, ldroot);
+    if (e == cudaSuccess && !fwd) apply_q(g, t, vec, ldv, nc, false, st);
+    return e;
+  };
+  for (int h = 0; h < g.H; ++h) TRY(sweep(h, true));
+  const Level64 root = root_level(g);
+  TRY(fwd_level64(root, g.rootvec, ldroot, g.rootz, ldroot, nullptr, 0, nc, st, log));
+  TRY(bwd_level64(root, g.rootvec, ldroot, g.rootz, ldroot, nullptr, 0, nc, st, log));
+  for (int h = g.H - 1; h >= 0; --h) TRY(sweep(h, false));
   TRY(cudaGetLastError());
   return HSS_OK;
 }

@@ -435,17 +435,6 @@ double qapply_flops(int b, int r, int nrhs) { return (4.0 * b * r + 2.0 * r * r)
 enum { SPLIT_D = 1, SPLIT_U = 2, SPLIT_E = 4, SPLIT_S = 8, SPLIT_ALL = 15 };
 cudaError_t split_generators(hss_s* h, cudaStream_t st, int which, bool lo);
 
-// Whether the Householder basis completion runs as panels and level-wide products.
-// In FP64 from the second 16-column panel on (level of 256 x 128 bases, any node
-// count up to the SMs: 2.7 -> 1.45 ms; 512 leaves of 512 x 128: 18.9 -> 8.4 ms; 16 of
-// 256 x 32: 0.29 -> 0.24 ms).  In FP32 the one-CTA kernel's products are fast and the
-// launches count: rank 96 loses 2 % of a step, rank 256 gains (leaf 1024: 8.9 ->
-// 3.1 ms, the levels above 2.2 -> 1.3 ms).
-template <typename T>
-bool ql_blocked(int r) {
-  return r > (sizeof(T) == 8 ? 16 : 128);
-}
-
 // levels L .. 1 of Alg. 2; leaves the merged root block in f.lv[0].A.
 // Two chains: the basis chain (basis completion of level l, then the merge's
 // rescaled coupling Ŝ and the parent basis, which need only L_B of level l) runs
@@ -567,8 +556,8 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
     if (c == 0 && cudaMemsetAsync(slots, 0, sizeof(double) * n, st) != cudaSuccess)
       return HSS_ERR_CUDA;
     if constexpr (std::is_same<T, double>::value) {
-      HSS_TRY(chol_level64({n, b, c, P.M, P.Li}, f.P, slots, l, 0, h->status, Q.A, ldq, sq, st,
-                           LaunchLog{h, st}));
+      HSS_TRY(chol_level64({n, b, c, P.M, P.Li}, f.P, slots, l, 0, h->status, {Q.A, ldq, sq, n},
+                           st, LaunchLog{h, st}));
     } else {
       // FP32: per panel of kPanel columns a per-node panel kernel (diagonal block
       // and the rows below it) and one SYRK of every node's trailing lower triangle
@@ -636,8 +625,8 @@ int factorize(hss_s* h, int prec, cudaStream_t st) {
     root = h->R0;
   }
   // root Cholesky (last step of Alg. 2), FP64 in every mode
-  HSS_TRY(chol_level64(root_level(h, root), h->f64.P, h->logdet_part, 0, 0, h->status, nullptr, 0,
-                       0, st, LaunchLog{h, st}));
+  HSS_TRY(chol_level64(root_level(h, root), h->f64.P, h->logdet_part, 0, 0, h->status, {}, st,
+                       LaunchLog{h, st}));
   {
     Launch k(h, HSS_K_OTHER, (double)((2LL << L) - 1), st);
     launch_logdet_reduce(h->logdet_part, (int)((2LL << L) - 1), h->logdet_val, st);

@@ -38,6 +38,21 @@ struct Level64 {
   int n, b, c;
   double* M;    // n x b x b, the factored blocks
   double* Li;   // n x inv_size(c), the inverted diagonal blocks
+
+  Level64 part(int first, int count) const {
+    return {count, b, c, M + (long long)first * b * b, Li + (long long)first * inv_size(c)};
+  }
+};
+
+// Where the merge puts a level's Schur complements: the diagonal blocks of the
+// parents PA (ld, stride) for the first `split` nodes, and those of PA2 for the
+// others (a forest's trees whose roots come next).  split is even.
+struct Merge64 {
+  double* PA = nullptr;
+  int ld = 0;
+  long long stride = 0;
+  int split = 0;
+  double* PA2 = nullptr;
 };
 
 // C (m x n) = alpha op(A) B + beta Cin, nc columns
@@ -63,12 +78,11 @@ inline cudaError_t skinny(int m, int nc, int k, const double* A, int lda, long l
 // then one update of the trailing triangle with 128 inner indices -- a whole
 // scaling group of the sliced product, which at 32 inner indices spends most of
 // its time putting the digits' sums together (512 nodes, order 480: 1.45 ms for 32,
-// 1.4 ms for 128).  The last update merges into the parents PA where given.
+// 1.4 ms for 128).  The last update merges into the parents where given.
 // P: scratch of n b 64 doubles.  log(kind, flops, fn) runs fn, one launch.
 template <typename Log>
 cudaError_t chol_level64(const Level64& lv, double* P, double* part, int level, int node0,
-                         int* status, double* PA, int ldpa, long long sPA, cudaStream_t st,
-                         const Log& log) {
+                         int* status, const Merge64& up, cudaStream_t st, const Log& log) {
   const int b = lv.b, c = lv.c, n = lv.n, lb = inv_order(c);
   const long long bb = (long long)b * b, sX = inv_size(c);
   for (int k0 = 0; k0 < c; k0 += kInvOrder) {
@@ -97,11 +111,23 @@ cudaError_t chol_level64(const Level64& lv, double* P, double* part, int level, 
     double* Mk = lv.M + k0 + (long long)k0 * b;
     const int rows = b - k0 - kb;
     if (rows > 0) {
-      double* C = Mk + kb + (long long)kb * b;
-      LV_TRY(HSS_K_SYR2K, (double)rows * (rows + 1.0) * kb * n,
-             (dsyrk_lower_batched(rows, kb, C, b, bb, Mk + kb, b, bb, C, b, bb,
-                                  k0 + kb == c ? PA : nullptr, ldpa, sPA, n, st),
-              cudaGetLastError()));
+      auto update = [&](int first, int count, double* PA) {
+        double* L = Mk + kb + first * bb;
+        double* C = L + (long long)kb * b;
+        LV_TRY(HSS_K_SYR2K, (double)rows * (rows + 1.0) * kb * count,
+               (dsyrk_lower_batched(rows, kb, C, b, bb, L, b, bb, C, b, bb, PA, up.ld, up.stride,
+                                    count, st),
+                cudaGetLastError()));
+        return cudaSuccess;
+      };
+      cudaError_t e = cudaSuccess;
+      if (k0 + kb < c || !(up.PA || up.PA2)) {
+        e = update(0, n, nullptr);
+      } else {
+        if (up.split > 0) e = update(0, up.split, up.PA);
+        if (e == cudaSuccess && n > up.split) e = update(up.split, n - up.split, up.PA2);
+      }
+      if (e != cudaSuccess) return e;
     }
     if (kb > 64) {   // off-diagonal block of the inverse: -X22 (L21 X11)
       const int k2 = kb - 64;

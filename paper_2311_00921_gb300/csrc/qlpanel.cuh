@@ -26,7 +26,17 @@ cudaError_t launch_ql_panel(const T* B, T* W, T* V, T* Tm, T* LB, int b, int r, 
 template <typename T>
 cudaError_t launch_ql_tblocks(const T* G, T* Tm, int r, int nodes, cudaStream_t st);
 
-// scratch: W b r, W1 and W2 r r, elements per node (r >= 1)
+// Whether the Householder basis completion runs as panels and level-wide products.
+// In FP64 from the second 16-column panel on (level of 256 x 128 bases, any node
+// count up to the SMs: 2.7 -> 1.45 ms; 512 leaves of 512 x 128: 18.9 -> 8.4 ms; 16 of
+// 256 x 32: 0.29 -> 0.24 ms).  In FP32 the one-CTA kernel's products are fast and the
+// launches count: rank 96 loses 2 % of a step, rank 256 gains (leaf 1024: 8.9 ->
+// 3.1 ms, the levels above 2.2 -> 1.3 ms).
+template <typename T>
+bool ql_blocked(int r) {
+  return r > (sizeof(T) == 8 ? 16 : 128);
+}
+
 template <typename T>
 void level_gemm(bool ta, bool tb, int m, int n, int k, T alpha, const T* A, int lda, long long sA,
                 const T* B, int ldb, long long sB, T beta, T* C, int ldc, long long sC, int batch,
@@ -49,7 +59,8 @@ inline int ql_panel_width(size_t elem, int b, int panel) {
   return elem == 8 || panel == 16 || b > 768 ? 16 : 32;
 }
 
-// V, L_B and the panels' blocks of T for n nodes of a level.  Right-looking: after
+// V, L_B and the panels' blocks of T for n nodes of a level (scratch per node: W
+// b r, W1 and W2 r r elements).  Right-looking: after
 // a panel, the later columns get A -= V_p (T_pᵀ V_pᵀ A) as three products.
 template <typename T, typename Log>
 cudaError_t ql_level(const T* B, T* V, T* Tm, T* LB, int b, int r, int n, T* W, T* W1, T* W2,

@@ -16,8 +16,6 @@
 //                         level eliminates nothing (rank = block order); otherwise
 //                         the last Schur update writes the parent block itself
 //                         (syrk_lower_merge_batched, gemm.cu).
-//  * pchol_kernel      -- the whole partial Cholesky of a node in one CTA, with
-//                         the merge as its epilogue (the batched forest path).
 //  * trsv_fwd_kernel /
 //    trsv_bwd_kernel   -- one level of the ULV solve (Sec. 3.2): forward
 //                         y := Qᵀ y (optionally), z^R = L^RR⁻¹ y^R, y^S -= L^SR z^R
@@ -396,148 +394,6 @@ ql_basis_kernel(const T* __restrict__ Bsrc, int ldb_src, long long sB, T* V, lon
     const T v2 = i2 > j ? w2 : (i2 == j ? T(1) : T(0));   // Ṽ(i2, j) -> V(i, j)
     W[i + (long long)j * b] = v2;
     if (i2 != i) W[i2 + (long long)j * b] = v1;
-  }
-}
-
-// ------------------------------------------------------------------ partial Cholesky
-template <typename T>
-__global__ void __launch_bounds__(NT)
-pchol_kernel(T* Mb, int ldm, long long sM, int b, int c, T* PA, int ldpa, long long sPA,
-             double* logdet_part, int level, int node0, int* status) {
-  extern __shared__ unsigned char smem_raw[];
-  T* P = reinterpret_cast<T*>(smem_raw);   // panel: b rows x NB, column-major ld = b
-  __shared__ int fail;
-  __shared__ double ld_acc;
-  const int node = blockIdx.x;
-  T* M = Mb + (long long)node * sM;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (tid == 0) {
-    fail = 0;
-    ld_acc = 0.0;
-  }
-  __syncthreads();
-
-  for (int k0 = 0; k0 < c; k0 += NB) {
-    const int kb = min(NB, c - k0);
-    const int n1 = b - k0;
-    // load panel M[k0:b, k0:k0+kb]
-    for (int e = tid; e < n1 * kb; e += NT) {
-      const int i = e % n1, jj = e / n1;
-      P[i + jj * b] = M[(k0 + i) + (long long)(k0 + jj) * ldm];
-    }
-    __syncthreads();
-    // diagonal block: one warp, lane i owns row i
-    if (wid == 0) {
-      double lsum = 0.0;
-      for (int jj = 0; jj < kb; ++jj) {
-        const T d = P[jj + jj * b];
-        if (!(d > T(0))) {
-          if (lane == 0) {
-            fail = 1;
-            report_failure(status, -3 /*NOT_SPD*/, level, node0 + node, k0 + jj);
-          }
-          break;
-        }
-        const T s = sqrt(d);
-        lsum += log((double)s);
-        __syncwarp();
-        if (lane > jj && lane < kb) P[lane + jj * b] /= s;
-        if (lane == jj) P[jj + jj * b] = s;
-        __syncwarp();
-        if (lane > jj && lane < kb) {
-          const T lij = P[lane + jj * b];
-          for (int t = jj + 1; t <= lane; ++t) P[lane + t * b] -= lij * P[t + jj * b];
-        }
-        __syncwarp();
-      }
-      if (lane == 0) ld_acc += lsum;
-    }
-    __syncthreads();
-    if (fail) return;
-    // panel TRSM: rows kb..n1-1 solve x L_diagᵀ = m, right-looking on a row held
-    // in registers (critical path kb steps, independent updates within a step)
-    for (int i = kb + tid; i < n1; i += NT) {
-      T x[NB];
-#pragma unroll
-      for (int jj = 0; jj < NB; ++jj) x[jj] = jj < kb ? P[i + jj * b] : T(0);
-#pragma unroll
-      for (int jj = 0; jj < NB; ++jj) {
-        if (jj < kb) {
-          x[jj] = x[jj] / P[jj + jj * b];
-#pragma unroll
-          for (int t = jj + 1; t < NB; ++t)
-            if (t < kb) x[t] = fma(-x[jj], P[t + jj * b], x[t]);
-        }
-      }
-#pragma unroll
-      for (int jj = 0; jj < NB; ++jj)
-        if (jj < kb) P[i + jj * b] = x[jj];
-    }
-    __syncthreads();
-    // write the panel back (lower part of the diagonal block and everything below)
-    for (int e = tid; e < n1 * kb; e += NT) {
-      const int i = e % n1, jj = e / n1;
-      if (i >= jj) M[(k0 + i) + (long long)(k0 + jj) * ldm] = P[i + jj * b];
-    }
-    // trailing update of the lower triangle, rows/cols >= k0 + kb
-    const int base = kb;   // panel row of the first trailing index
-    const int n2 = n1 - kb;
-    if (n2 > 0) {
-      const int nt = (n2 + 63) / 64;
-      const int tx = tid & 15, ty = tid >> 4;
-      for (int tp = 0; tp < nt * (nt + 1) / 2; ++tp) {
-        int t = tp, ti = 0;
-        while (t > ti) { t -= ti + 1; ++ti; }
-        const int tj = t;
-        T acc[4][4];
-#pragma unroll
-        for (int p = 0; p < 4; ++p)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) acc[p][q] = T(0);
-        for (int kk = 0; kk < kb; ++kk) {
-          T a[4], bb[4];
-#pragma unroll
-          for (int s = 0; s < 4; ++s) {
-            const int ri = ti * 64 + tx + 16 * s;
-            const int rj = tj * 64 + ty + 16 * s;
-            a[s] = ri < n2 ? P[base + ri + kk * b] : T(0);
-            bb[s] = rj < n2 ? P[base + rj + kk * b] : T(0);
-          }
-#pragma unroll
-          for (int p = 0; p < 4; ++p)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[p][q] = fma(a[p], bb[q], acc[p][q]);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int rj = tj * 64 + ty + 16 * q;
-          if (rj >= n2) continue;
-#pragma unroll
-          for (int p = 0; p < 4; ++p) {
-            const int ri = ti * 64 + tx + 16 * p;
-            if (ri >= n2 || ri < rj) continue;
-            T* m = M + (k0 + kb + ri) + (long long)(k0 + kb + rj) * ldm;
-            *m -= acc[p][q];
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && logdet_part) logdet_part[node0 + node] = 2.0 * ld_acc;
-  // merge epilogue: Â^SS (r x r, lower) -> parent diagonal block at (off, off)
-  if (PA) {
-    const int r = b - c;
-    const int p = node >> 1;
-    const int off = (node & 1) * r;
-    T* A = PA + (long long)p * sPA;
-    for (int e = tid; e < r * r; e += NT) {
-      const int i = e % r, j = e / r;
-      if (i < j) continue;
-      const T v = M[(c + i) + (long long)(c + j) * ldm];
-      A[(off + i) + (long long)(off + j) * ldpa] = v;
-      A[(off + j) + (long long)(off + i) * ldpa] = v;
-    }
   }
 }
 
@@ -1380,20 +1236,6 @@ cudaError_t launch_ql_basis(const T* Bsrc, int ldb_src, long long sB, T* V, long
 }
 
 template <typename T>
-size_t pchol_smem(int b) { return (size_t)b * NB * sizeof(T); }
-
-template <typename T>
-cudaError_t launch_pchol(T* M, int ldm, long long sM, int b, int c, T* PA, int ldpa, long long sPA,
-                         double* logdet_part, int level, int node0, int* status, int nodes,
-                         cudaStream_t st) {
-  const size_t sm = pchol_smem<T>(b);
-  if (!smem_opt_in(pchol_kernel<T>, sm)) return cudaErrorInvalidConfiguration;
-  pchol_kernel<T><<<nodes, NT, sm, st>>>(M, ldm, sM, b, c, PA, ldpa, sPA, logdet_part, level,
-                                         node0, status);
-  return cudaGetLastError();
-}
-
-template <typename T>
 cudaError_t launch_chol_panel(T* M, int ldm, long long sM, int rows, int kb, double* logdet_part,
                               int level, int node0, int col0, int* status, int nodes,
                               bool accumulate, cudaStream_t st, int splits) {
@@ -1625,22 +1467,6 @@ cudaError_t launch_tree_bwd(const TreeLevels<T>& lv, int lo, int b, int c, int r
                                      args, sm, st);
 }
 
-template <typename T>
-cudaError_t launch_trsv_fwd(const T* M, int ldm, long long sM, int b, int c, T* X, int ldx,
-                            long long sX, int nrhs, T* Par, int ldpar, long long sPar, int nodes,
-                            cudaStream_t st) {
-  return launch_ulv_fwd<T>(M, ldm, sM, b, c, X, ldx, sX, nrhs, Par, ldpar, sPar, nullptr, 0,
-                           nullptr, 0, 0, nodes, st, 0);
-}
-
-template <typename T>
-cudaError_t launch_trsv_bwd(const T* M, int ldm, long long sM, int b, int c, T* X, int ldx,
-                            long long sX, int nrhs, const T* Par, int ldpar, long long sPar,
-                            int nodes, cudaStream_t st) {
-  return launch_ulv_bwd<T>(M, ldm, sM, b, c, X, ldx, sX, nrhs, Par, ldpar, sPar, nullptr, 0,
-                           nullptr, 0, 0, nodes, st, 0);
-}
-
 void launch_logdet_reduce(const double* part, int n, double* out, cudaStream_t st) {
   logdet_reduce_kernel<<<1, 1024, 0, st>>>(part, n, out);
 }
@@ -1649,12 +1475,6 @@ void launch_logdet_reduce(const double* part, int n, double* out, cudaStream_t s
   template cudaError_t launch_ql_basis<T>(const T*, int, long long, T*, long long, T*, long long,  \
                                           T*, long long, int, int, int, cudaStream_t,             \
                                           const int*, int);                                        \
-  template cudaError_t launch_pchol<T>(T*, int, long long, int, int, T*, int, long long, double*, \
-                                       int, int, int*, int, cudaStream_t);                        \
-  template cudaError_t launch_trsv_fwd<T>(const T*, int, long long, int, int, T*, int, long long, \
-                                          int, T*, int, long long, int, cudaStream_t);            \
-  template cudaError_t launch_trsv_bwd<T>(const T*, int, long long, int, int, T*, int, long long, \
-                                          int, const T*, int, long long, int, cudaStream_t);      \
   template cudaError_t launch_ulv_fwd<T>(const T*, int, long long, int, int, T*, int, long long,  \
                                          int, T*, int, long long, const T*, long long, const T*,  \
                                          long long, int, int, cudaStream_t, int);                 \

@@ -16,26 +16,9 @@ cudaError_t launch_ql_basis(const T* Bsrc, int ldb_src, long long sB, T* V, long
 // blocked completion has no such limit but keeps to the documented one.
 bool ql_accepts64(int b, int r);
 
-template <typename T>
-size_t pchol_smem(int b);
-
-template <typename T>
-cudaError_t launch_pchol(T* M, int ldm, long long sM, int b, int c, T* PA, int ldpa, long long sPA,
-                  double* logdet_part, int level, int node0, int* status, int nodes,
-                  cudaStream_t st);
-
-template <typename T>
-cudaError_t launch_trsv_fwd(const T* M, int ldm, long long sM, int b, int c, T* X, int ldx, long long sX,
-                     int nrhs, T* Par, int ldpar, long long sPar, int nodes, cudaStream_t st);
-
-template <typename T>
-cudaError_t launch_trsv_bwd(const T* M, int ldm, long long sM, int b, int c, T* X, int ldx, long long sX,
-                     int nrhs, const T* Par, int ldpar, long long sPar, int nodes,
-                     cudaStream_t st);
-
 // One level of the ULV solve per launch, one CTA per node: the forward sweep
 // applies Qᵀ = I - V Tᵀ Vᵀ to the node segment and then the triangular forward
-// sweep (launch_trsv_fwd); the backward sweep runs the triangular backward sweep
+// sweep; the backward sweep runs the triangular backward sweep
 // and then applies Q = I - V T Vᵀ.  V (b x r, batch stride sV) and T (r x r,
 // batch stride sT) are the node's compact-WY basis (Eq. 2-3); V = null skips
 // the Q application.  nrhs <= 16, r <= min(b, 256).  staging: 0 = the
