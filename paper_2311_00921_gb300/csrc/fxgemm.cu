@@ -385,6 +385,203 @@ fx_gemm_kernel(const __grid_constant__ FxShape s) {
     }
 }
 
+// ------------------------------------------------------------------ narrow products
+// n <= 16 columns (right-hand sides; B's inner index contiguous), a CTA 16 rows and
+// every column.  The four warps of a team take 32 inner indices each of a group of
+// 128, hold them as the MMA's fragments (inner index kw + 16 q + t + 4 j for lane t of
+// a quad, in both operands) and convert them in registers: every operand element is
+// read once, and the row maxima are the only thing the warps exchange before the
+// MMAs.  The team's accumulators, exact integers up to 2^24, are then added through
+// shared memory, each warp putting a quarter of the sums together.  TEAMS = 2: two
+// groups at a time.  At the sizes of the upper levels a launch is one such chain, bound
+// by its latency: a 128 x 256 node and 16 columns 8.4 us where fx_gemm_kernel, which
+// reads the strips twice and passes them through shared memory, takes 24.7 us.
+template <int NB, int TEAMS>
+constexpr int skinny_smem() {
+  return TEAMS * 4 * (4 * NB) * 2 * 32 * (int)sizeof(float4);
+}
+
+template <int NB, int TEAMS, bool AKC>
+__global__ void __launch_bounds__(128 * TEAMS, (NB == 1 ? 4 : 2) / TEAMS)
+fx_skinny_kernel(const __grid_constant__ FxShape s) {
+  constexpr int R = 16, BN = 8 * NB, E = 4 * NB;   // E: fragment registers
+  extern __shared__ __align__(16) float4 xch[];    // [team][warp][E][2][lane]
+  __shared__ int mx[TEAMS][4][R + BN];
+  const int tid = threadIdx.x, lane = tid & 31, w = (tid >> 5) & 3, team = tid >> 7;
+  const int g = lane >> 2, t = lane & 3;
+  const long long z = blockIdx.x / s.tiles;
+  const int i0 = (int)(blockIdx.x % s.tiles) * R;
+  const double* A = s.a.p1 + z * s.a.s1;
+  const double* B = s.b.p1 + z * s.b.s1;
+  const long long lda = s.a.ld1, ldb = s.b.ld1;
+  // rows and columns past the last are read as copies of it: not stored
+  const double *pa[2], *pb[NB];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int i = min(i0 + 8 * h + g, s.m - 1);
+    pa[h] = A + (AKC ? i * lda : i);
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b) pb[b] = B + min(8 * b + g, s.n - 1) * ldb;
+
+  double res[NB];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) res[b] = 0.0;
+
+  for (int kt = 0; kt < s.K; kt += kGroup * TEAMS) {
+    const int kg = kt + kGroup * team, ke = min(s.K, kg + kGroup), kw = kg + 32 * w;
+    double av[2][2][4], bv[NB][2][4];   // [half of the rows or block, half of 32 indices, j]
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int k = kw + 16 * q + t + 4 * j;
+        const bool in = k < ke;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) av[h][q][j] = in ? pa[h][AKC ? (long long)k : k * lda] : 0.0;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) bv[b][q][j] = in ? pb[b][k] : 0.0;
+      }
+    auto quad_max = [&](const double (&v)[2][4]) {   // over the quad's 32 indices
+      int x = 0;
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x = max(x, __double2hiint(v[q][j]) & 0x7fffffff);
+      x = max(x, __shfl_xor_sync(0xffffffffu, x, 1));
+      return max(x, __shfl_xor_sync(0xffffffffu, x, 2));
+    };
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int x = quad_max(av[h]);
+      if (t == 0) mx[team][w][8 * h + g] = x;
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const int x = quad_max(bv[b]);
+      if (t == 0) mx[team][w][R + 8 * b + g] = x;
+    }
+    __syncthreads();
+    int odd = 0;
+    auto exponent = [&](int r) {   // as in fx_gemm_kernel
+      const int h = max(max(mx[team][0][r], mx[team][1][r]), max(mx[team][2][r], mx[team][3][r]));
+      odd |= h >= kHiBig || (h > 0 && h < kHiSmall);
+      return (h ? (h + 0x2100) >> 20 : 1023) + 1;
+    };
+    int ea[2], eb[NB];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) ea[h] = exponent(8 * h + g);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) eb[b] = exponent(R + 8 * b + g);
+    const bool plain = __any_sync(0xffffffffu, odd);   // the same in the team's warps
+    float acc[kDigits][NB][4];
+#pragma unroll
+    for (int d = 0; d < kDigits; ++d)
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[d][b][e] = 0.f;
+    if (!plain) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        if (kw + 16 * q < ke) {
+          uint32_t bd[NB][2][kDigits], ad[4][kDigits];
+#pragma unroll
+          for (int b = 0; b < NB; ++b)
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+              digits(fixed_point(bv[b][q][2 * p], eb[b]), fixed_point(bv[b][q][2 * p + 1], eb[b]),
+                     bd[b][p]);
+#pragma unroll
+          for (int p = 0; p < 4; ++p)   // fragment register p: row half p & 1, indices p >> 1
+            digits(fixed_point(av[p & 1][q][2 * (p >> 1)], ea[p & 1]),
+                   fixed_point(av[p & 1][q][2 * (p >> 1) + 1], ea[p & 1]), ad[p]);
+#pragma unroll
+          for (int i = 0; i < kDigits; ++i) {
+            const uint32_t a[4] = {ad[0][i], ad[1][i], ad[2][i], ad[3][i]};
+#pragma unroll
+            for (int j = 0; i + j < kDigits; ++j)
+#pragma unroll
+              for (int b = 0; b < NB; ++b) mma_f16(acc[i + j][b], a, bd[b][0][j], bd[b][1][j]);
+          }
+        }
+      }
+    }
+    float4* mine = xch + (team * 4 + w) * (E * 64) + lane;
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          mine[((b * 4 + e) * 2 + h) * 32] = make_float4(acc[4 * h][b][e], acc[4 * h + 1][b][e],
+                                                         acc[4 * h + 2][b][e], acc[4 * h + 3][b][e]);
+    __syncthreads();
+    // warp w: fragment register w of every block, row g + 8 (w >> 1), column 2 t + (w & 1)
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const int ex =
+          __shfl_sync(0xffffffffu, eb[b], (2 * t + (w & 1)) * 4) + (w & 2 ? ea[1] : ea[0]);
+      if (!plain) {
+        long long v[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const float4 y = xch[(team * 4 + u) * (E * 64) + ((b * 4 + w) * 2 + h) * 32 + lane];
+            x.x += y.x, x.y += y.y, x.z += y.z, x.w += y.w;
+          }
+          v[h] = (long long)__float2int_rn(x.x) * (1 << 24) +
+                 (long long)__float2int_rn(x.y) * (1 << 16) +
+                 (long long)__float2int_rn(x.z) * (1 << 8) + __float2int_rn(x.w);
+        }
+        const double scale = __hiloint2double((ex - 1093) << 20, 0);
+        res[b] = fma(fma((double)v[0], 4294967296.0, (double)v[1]), scale, res[b]);
+      } else {   // plain FP64 for this group
+        const int i = min(i0 + 8 * (w >> 1) + g, s.m - 1);
+        const int j = min(8 * b + 2 * t + (w & 1), s.n - 1);
+        for (int k = kg; k < ke; ++k)
+          res[b] = fma(A[AKC ? i * lda + k : i + k * lda], B[j * ldb + k], res[b]);
+      }
+    }
+  }
+
+  if (TEAMS > 1) {
+    double* sum = reinterpret_cast<double*>(xch);
+    __syncthreads();
+    if (team == 1) {
+#pragma unroll
+      for (int b = 0; b < NB; ++b) sum[b * 128 + (tid & 127)] = res[b];
+    }
+    __syncthreads();
+    if (team == 1) return;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) res[b] += sum[b * 128 + tid];
+  }
+  double* C = s.C + z * s.sC;
+  const double* Ci = s.Cin + z * s.sCin;
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const int i = i0 + 8 * (w >> 1) + g, j = 8 * b + 2 * t + (w & 1);
+    if (i >= s.m || j >= s.n) continue;
+    double v = s.alpha * res[b];
+    if (s.beta != 0.0) v = fma(s.beta, Ci[i + (long long)j * s.ldcin], v);
+    C[i + (long long)j * s.ldc] = v;
+  }
+}
+
+template <int NB, int TEAMS>
+cudaError_t launch_skinny(FxShape& s, int batch, cudaStream_t st) {
+  s.tiles = (s.m + 15) / 16;
+  const auto kernel = s.a.kc ? fx_skinny_kernel<NB, TEAMS, true> : fx_skinny_kernel<NB, TEAMS, false>;
+  const int bytes = skinny_smem<NB, TEAMS>();
+  const cudaError_t e = fx_allow_smem(reinterpret_cast<const void*>(kernel), bytes);
+  if (e != cudaSuccess) return e;
+  kernel<<<(unsigned)((long long)s.tiles * batch), 128 * TEAMS, bytes, st>>>(s);
+  return cudaGetLastError();
+}
+
 template <int BN, bool AKC, bool BKC>
 cudaError_t launch(FxShape& s, int batch, cudaStream_t st) {
   s.tiles_m = (s.m + kRows - 1) / kRows;
@@ -434,6 +631,21 @@ cudaError_t fx_gemm(int m, int n, int K, const FxOperand& a, const FxOperand& b,
                     cudaStream_t st) {
   FxShape s{m, n, K, a.p2 ? K / 2 : K, a, b, alpha, beta, Cin ? Cin : C, ldcin, sCin, C, ldc, sC, lower ? 1 : 0,
             PA, ldpa, sPA, 0, 0, 0};
+  // Narrow products (B's inner index contiguous).  Up to 8 columns fx_skinny_kernel is
+  // the faster one at every size (512 x 512, 512 nodes: 481 against 506 us; 128 nodes:
+  // 128 against 150; 128 x 128, 8 nodes: 6.2 against 10.5).  With 9 to 16 it wins while
+  // the 64-row tiles of the other kernel leave SMs idle (128 x 256, 16 nodes: 8.4
+  // against 24.7 us; 33 nodes 12.5 against 22.7), and loses where they fill the chip (256
+  // nodes: 62 against 57; 512 x 512, 512 nodes: 950 against 660): there the 64 rows
+  // share one conversion of B.  Two groups at a time while a wave of CTAs takes them
+  // all (8 nodes of 128 x 256, 8 columns: 6.3 against 8.2 us; 264 tiles: 14.5
+  // against 12.5).
+  if (n <= 16 && b.kc && !a.p2 && !lower) {
+    const bool two = K > kGroup && (long long)((m + 15) / 16) * batch <= 152;
+    if (n <= 8) return two ? launch_skinny<1, 2>(s, batch, st) : launch_skinny<1, 1>(s, batch, st);
+    if ((long long)((m + kRows - 1) / kRows) * batch <= 304)
+      return two ? launch_skinny<2, 2>(s, batch, st) : launch_skinny<2, 1>(s, batch, st);
+  }
   if (n <= 8) return launch_modes<8>(s, batch, st);
   if (n <= 16) return launch_modes<16>(s, batch, st);
   return launch_modes<32>(s, batch, st);

@@ -114,3 +114,32 @@ def test_pivot_in_a_later_block():
     assert (info["level"], info["node"], info["col"]) == (eo.value.level, eo.value.node,
                                                          eo.value.col)
     assert info["col"] > 64
+
+
+@pytest.mark.parametrize("leaf,rank,nrhs", [
+    (1, 1, 8), (15, 15, 9), (16, 7, 16), (17, 17, 1), (127, 33, 8), (128, 4, 7), (257, 40, 3),
+    (1300, 5, 8), (1300, 5, 16), (2500, 2, 8)])
+def test_narrow_products_against_extended_precision(leaf, rank, nrhs):
+    """Right-hand sides of up to 8 and 16 columns at the edges of the narrow kernel's
+    tiles (16 rows, 32 indices a warp, one and two groups at a time)."""
+    test_products_against_extended_precision(leaf, rank, nrhs, 6)
+
+
+def test_batch_levels_against_oracle():
+    """A forest whose heights hold both kinds of parents, at ranks below, at and above
+    the blocks of the level routines, with nothing eliminated at some leaves."""
+    from oracle import ulv as O
+    from paper_2311_00921_gb300 import inputs as I
+    mats = [I.random_hss(L, leaf, r, seed=50 + i, orthonormal=False) for i, (L, leaf, r) in
+            enumerate([(3, 90, 17), (1, 90, 17), (2, 90, 17), (2, 24, 24), (1, 24, 24),
+                       (2, 200, 130), (1, 200, 130), (2, 300, 9)])]
+    bs = [I.rhs(h.n, 3, 60 + i) for i, h in enumerate(mats)]
+    bt = hss.HSSBatch(mats)
+    bt.factorize()
+    xs, lds = bt.solve([hss.colmajor(b) for b in bs]), bt.logdet()
+    for h, b, x, ld in zip(mats, bs, xs, lds):
+        F = O.factor(h)
+        x_ref, ld_ref = O.solve(F, b), O.logdet(F)
+        err = np.linalg.norm(x.cpu().numpy() - x_ref, axis=0) / np.linalg.norm(x_ref, axis=0)
+        assert err.max() <= 1e-10
+        assert abs(ld - ld_ref) <= 1e-12 * abs(ld_ref)
