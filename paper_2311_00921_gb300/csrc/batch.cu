@@ -326,8 +326,8 @@ int solve_group(Group& g, int nc) {
     auto part = [&](int first, int count, double* par, int ldpar) {
       double *y = vec + (long long)first * t.b, *z = t.zv + (long long)first * t.b;
       const Level64 lv = t.level().part(first, count);
-      return fwd ? fwd_level64(lv, y, ldv, z, ldz, par, ldpar, nc, st, log)
-                 : bwd_level64(lv, y, ldv, z, ldz, par, ldpar, nc, st, log);
+      return fwd ? fwd_level(lv, y, ldv, z, ldz, par, ldpar, nc, st, log)
+                 : bwd_level(lv, y, ldv, z, ldz, par, ldpar, nc, st, log);
     };
     if (fwd) apply_q(g, t, vec, ldv, nc, true, st);
     cudaError_t e = cudaSuccess;
@@ -342,8 +342,8 @@ int solve_group(Group& g, int nc) {
   };
   for (int h = 0; h < g.H; ++h) TRY(sweep(h, true));
   const Level64 root = root_level(g);
-  TRY(fwd_level64(root, g.rootvec, ldroot, g.rootz, ldroot, nullptr, 0, nc, st, log));
-  TRY(bwd_level64(root, g.rootvec, ldroot, g.rootz, ldroot, nullptr, 0, nc, st, log));
+  TRY(fwd_level<double>(root, g.rootvec, ldroot, g.rootz, ldroot, nullptr, 0, nc, st, log));
+  TRY(bwd_level<double>(root, g.rootvec, ldroot, g.rootz, ldroot, nullptr, 0, nc, st, log));
   for (int h = g.H - 1; h >= 0; --h) TRY(sweep(h, false));
   TRY(cudaGetLastError());
   return HSS_OK;

@@ -34,7 +34,8 @@ namespace {
 constexpr int kMaxCols = 32;      // right-hand-side columns per matvec pass
 constexpr int kSolveCols = 16;    // columns per triangular-sweep / refinement pass
 constexpr int kPanel = 32;        // columns per blocked-Cholesky panel (the panel kernel's limit)
-constexpr int kTreeRank = 16;     // FP64 solves up to this rank run on the per-node kernels
+constexpr int kTreeRank = 16;     // FP64 solves up to this rank run on the per-node kernels,
+constexpr int kTreeRank32 = 32;   // FP32 sweeps up to this one (see solve_levels)
 constexpr int kFuseNodes = 64;    // levels up to this many nodes apply Q inside the sweep kernel
 constexpr int kTreeTop = 6;       // levels 1 .. 6 (<= 64 nodes): one tree launch per direction
 
@@ -48,8 +49,8 @@ struct LevelT {
   T* A = nullptr;   // n x b x b merged blocks (levels < L), 1 block at the root
   T* B = nullptr;   // n x b x r bases fed to the QL (levels 1 .. L-1)
   T* yv = nullptr;  // level vector of the solve: (n b) x kSolveCols
-  T* Li = nullptr;  // FP64: inverted diagonal blocks of L^RR (chol64.cuh)
-  T* zv = nullptr;  // FP64: the forward sweep's z^R, laid out as yv
+  T* Li = nullptr;  // inverted diagonal blocks of L^RR (chol64.cuh)
+  T* zv = nullptr;  // the forward sweep's z^R, laid out as yv
 };
 
 template <typename T>
@@ -195,7 +196,7 @@ void layout_factor(Bump& bp, Factor<T>& f, int L, int leaf, int r) {
     }
     if (l >= 1 && l < L) P.B = bp.take<T>((size_t)P.n * P.b * r);
     if (l < L) P.yv = bp.take<T>((size_t)P.n * P.b * kSolveCols);
-    if (sizeof(T) == 8) {
+    if (sizeof(T) == 8 || (l >= 1 && r > kTreeRank32)) {
       P.Li = bp.take<T>((size_t)P.n * inv_size(P.c));
       P.zv = bp.take<T>((size_t)P.n * P.b * kSolveCols);
     }
@@ -507,6 +508,7 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
     if (rc) return rc;
   }
   // main chain
+  bool inverses = false;
   for (int l = L; l >= 1; --l) {
     LevelT<T>& P = f.lv[l];
     LevelT<T>& Q = f.lv[l - 1];
@@ -581,6 +583,18 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
         }
       }
     }
+    if constexpr (std::is_same<T, float>::value) {
+      // the sweeps' inverses, beside the next levels
+      if (r > kTreeRank32 && c > 0) {
+        const cudaStream_t is = h->serialize ? st : h->lane[0].ms;
+        if (cudaEventRecord(h->lane[0].mv_start, st) != cudaSuccess ||
+            cudaStreamWaitEvent(is, h->lane[0].mv_start, 0) != cudaSuccess)
+          return HSS_ERR_CUDA;
+        inverses = true;
+        Launch k(h, HSS_K_OTHER, (double)inv_order(c) * inv_order(c) * c / 3.0 * n, is, true);
+        HSS_TRY(launch_inv32(P.M, b, bb, c, P.Li, inv_size(c), n, is));
+      }
+    }
     // (d, second half) with nothing eliminated (c = 0) Â^SS is the whole block:
     // copied into the parents' diagonal blocks by its own pass
     if (c == 0) {
@@ -590,6 +604,10 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
     int rc = check_launch();
     if (rc) return rc;
   }
+  if (inverses && !h->serialize &&
+      (cudaEventRecord(h->lane[0].mv_dx, h->lane[0].ms) != cudaSuccess ||
+       cudaStreamWaitEvent(st, h->lane[0].mv_dx, 0) != cudaSuccess))
+    return HSS_ERR_CUDA;
   return HSS_OK;
 }
 
@@ -645,52 +663,86 @@ void apply_q(hss_s* h, Factor<T>& f, const LevelT<T>& P, T* vec, int ldv, int nc
   const long long s1 = (long long)r * kSolveCols;
   T* t1 = f.t1 + (long long)col0 * r;   // this lane's columns of the scratch
   T* t2 = f.t2 + (long long)col0 * r;
-  gemm<T>(h, true, false, r, nc, b, T(1), P.V, b, (long long)b * r, vec, ldv, b, T(0), t1, r, s1,
-          n, st);
-  gemm<T>(h, transpose, false, r, nc, r, T(1), P.T_, r, (long long)r * r, t1, r, s1, T(0), t2, r,
-          s1, n, st);
-  gemm<T>(h, false, false, b, nc, r, T(-1), P.V, b, (long long)b * r, t2, r, s1, T(1), vec, ldv,
-          b, n, st);
+  auto product = [&](bool ta, int m, int k, T alpha, const T* A, int lda, long long sA, const T* B,
+                     int ldb, long long sB, T beta, T* C, int ldc, long long sC) {
+    if constexpr (std::is_same<T, float>::value) {
+      Launch l(h, HSS_K_GEMM_SKINNY, 2.0 * m * nc * (double)k * n, st, true);
+      narrow32(m, nc, k, A, lda, sA, ta, B, ldb, sB, alpha, beta != 0.f ? C : nullptr, ldc, sC, C,
+               ldc, sC, n, st);   // launch errors: the callers' check
+    } else {
+      gemm<T>(h, ta, false, m, nc, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, n, st);
+    }
+  };
+  product(true, r, b, T(1), P.V, b, (long long)b * r, vec, ldv, b, T(0), t1, r, s1);
+  product(transpose, r, r, T(1), P.T_, r, (long long)r * r, t1, r, s1, T(0), t2, r, s1);
+  product(false, b, r, T(-1), P.V, b, (long long)b * r, t2, r, s1, T(1), vec, ldv, b);
 }
 
 // root solve on nc columns of y (2 rank rows), z: scratch of the same size
 int solve_root(hss_s* h, double* R, double* y, double* z, int nc, cudaStream_t st) {
   const int b0 = 2 * h->rank;
   const Level64 lv = root_level(h, R);
-  HSS_TRY(fwd_level64(lv, y, b0, z, b0, nullptr, 0, nc, st, LaunchLog{h, st}));
-  HSS_TRY(bwd_level64(lv, y, b0, z, b0, nullptr, 0, nc, st, LaunchLog{h, st}));
+  HSS_TRY(fwd_level<double>(lv, y, b0, z, b0, nullptr, 0, nc, st, LaunchLog{h, st}));
+  HSS_TRY(bwd_level<double>(lv, y, b0, z, b0, nullptr, 0, nc, st, LaunchLog{h, st}));
   return HSS_OK;
 }
 
-// The FP64 ULV sweeps as products over whole levels: Q by three, each triangular
-// sweep by two per 128 eliminated columns (chol64.cuh).  A node's sweep in one CTA
-// is bound by that SM's FP64 pipe, 540 us a level and direction at rank 128 with 16
-// columns (78 us at rank 32 with one) against 65 us (33 us) for the products; up
-// to rank kTreeRank the per-node kernels, one launch for all upper levels, are as
-// fast or faster and stay.
-int solve_levels64(hss_s* h, double* x, int nc, int ld, cudaStream_t st) {
-  const int L = h->L;
-  Factor<double>& f = h->f64;
-  const LaunchLog log{h, st};
-  auto level = [&](int l) {
-    const LevelT<double>& P = f.lv[l];
-    return Level64{P.n, P.b, P.c, P.M, P.Li};
-  };
-  for (int l = L; l >= 1; --l) {
-    const LevelT<double>&P = f.lv[l], &Q = f.lv[l - 1];
-    double* vec = l == L ? x : P.yv;
-    const int ldz = P.n * P.b, ldv = l == L ? ld : ldz;
-    apply_q<double>(h, f, P, vec, ldv, nc, /*transpose=*/true, st, 0);
-    HSS_TRY(fwd_level64(level(l), vec, ldv, P.zv, ldz, Q.yv, Q.n * Q.b, nc, st, log));
+// root solve of a sweep, FP64 in every mode: the root's vector is that of level 0
+template <typename T>
+int sweep_root(hss_s* h, Factor<T>& f, T* v0, int nc, int col0, cudaStream_t st) {
+  const int b0 = 2 * h->rank;
+  if constexpr (std::is_same<T, double>::value) {
+    return solve_root(h, f.lv[0].A, v0, f.lv[0].zv, nc, st);
+  } else {
+    const long long o = (long long)col0 * b0;
+    double* rv = h->root_vec + o;
+    {
+      Launch k(h, HSS_K_OTHER, 0.0, st);
+      launch_f32_to_f64(v0, rv, (long long)b0 * nc, st);
+    }
+    const int rc = solve_root(h, h->R0, rv, h->root_vec2 + o, nc, st);
+    if (rc) return rc;
+    Launch k(h, HSS_K_OTHER, 0.0, st);
+    launch_f64_to_f32(rv, v0, (long long)b0 * nc, st);
+    return HSS_OK;
   }
-  const int rc = solve_root(h, f.lv[0].A, f.lv[0].yv, f.lv[0].zv, nc, st);
+}
+
+// The ULV sweeps as products over whole levels: Q by three, each triangular sweep by
+// two per 128 eliminated columns (chol64.cuh).  A node's sweep in one CTA is in FP64
+// bound by that SM's pipe, 540 us a level and direction at rank 128 with 16 columns
+// (78 us at rank 32 with one) against 50 us (25 us) for the products; up to rank
+// kTreeRank the per-node kernels, one launch for all upper levels, are as fast or
+// faster and stay.  In FP32 it is a chain of 32-column steps: rank 128, 16 columns,
+// 151 us a level and direction on average of N = 262144 against 71, rank 96, 3 columns,
+// 50 against 22.  The line is at rank 32 there: N = 16384, one column, 1.06 ms by the
+// tree kernels and 1.15 by products at rank 32, 1.24 and 1.16 at rank 48.
+template <typename T>
+int solve_levels(hss_s* h, Factor<T>& f, T* x, int nc, int ld, cudaStream_t st, int col0) {
+  const int L = h->L;
+  const LaunchLog log{h, st, sizeof(T) == 4};
+  auto level = [&](int l) {
+    const LevelT<T>& P = f.lv[l];
+    return LevelOf<T>{P.n, P.b, P.c, P.M, P.Li};
+  };
+  // this lane's columns of a level's vectors
+  auto yv = [&](int l) { return f.lv[l].yv + (long long)col0 * f.lv[l].n * f.lv[l].b; };
+  auto zv = [&](int l) { return f.lv[l].zv + (long long)col0 * f.lv[l].n * f.lv[l].b; };
+  for (int l = L; l >= 1; --l) {
+    const LevelT<T>&P = f.lv[l], &Q = f.lv[l - 1];
+    T* vec = l == L ? x : yv(l);
+    const int ldz = P.n * P.b, ldv = l == L ? ld : ldz;
+    apply_q<T>(h, f, P, vec, ldv, nc, /*transpose=*/true, st, col0);
+    HSS_TRY(fwd_level<T>(level(l), vec, ldv, zv(l), ldz, yv(l - 1), Q.n * Q.b, nc, st, log));
+  }
+  const int rc = sweep_root<T>(h, f, yv(0), nc, col0, st);
   if (rc) return rc;
   for (int l = 1; l <= L; ++l) {
-    const LevelT<double>&P = f.lv[l], &Q = f.lv[l - 1];
-    double* vec = l == L ? x : P.yv;
+    const LevelT<T>&P = f.lv[l], &Q = f.lv[l - 1];
+    T* vec = l == L ? x : yv(l);
     const int ldz = P.n * P.b, ldv = l == L ? ld : ldz;
-    HSS_TRY(bwd_level64(level(l), vec, ldv, P.zv, ldz, Q.yv, Q.n * Q.b, nc, st, log));
-    apply_q<double>(h, f, P, vec, ldv, nc, /*transpose=*/false, st, 0);
+    HSS_TRY(bwd_level<T>(level(l), vec, ldv, zv(l), ldz, yv(l - 1), Q.n * Q.b, nc, st, log));
+    apply_q<T>(h, f, P, vec, ldv, nc, /*transpose=*/false, st, col0);
   }
   return check_launch();
 }
@@ -702,9 +754,8 @@ template <typename T>
 int solve_sweeps(hss_s* h, Factor<T>& f, T* x, int nc, int ld, cudaStream_t st, int g = 0,
                  int col0 = 0) {
   const int L = h->L, r = h->rank;
-  if constexpr (std::is_same<T, double>::value) {
-    if (r > kTreeRank) return solve_levels64(h, x, nc, ld, st);
-  }
+  if (r > (sizeof(T) == 8 ? kTreeRank : kTreeRank32))
+    return solve_levels<T>(h, f, x, nc, ld, st, col0);
   Lane& ln = h->lane[g];
   // level l's vector, this lane's columns
   auto lvec = [&](int l) { return f.lv[l].yv + (long long)col0 * f.lv[l].n * f.lv[l].b; };
@@ -744,27 +795,8 @@ int solve_sweeps(hss_s* h, Factor<T>& f, T* x, int nc, int ld, cudaStream_t st, 
     Launch k(h, HSS_K_TRSV_FWD, tree_flops, st, sizeof(T) == 4);
     HSS_TRY(launch_tree_fwd<T>(tl, lo, 2 * r, r, r, nc, ln.tcnt, st));
   }
-  const int b0 = 2 * r;
-  const long long rc0 = (long long)col0 * b0;
-  double* rootA;
-  double* rv;
-  if (sizeof(T) == sizeof(double)) {
-    rootA = reinterpret_cast<double*>(f.lv[0].A);
-    rv = reinterpret_cast<double*>(lvec(0));
-  } else {
-    rootA = h->R0;
-    rv = h->root_vec + rc0;
-    Launch k(h, HSS_K_OTHER, 0.0, st);
-    launch_f32_to_f64(reinterpret_cast<const float*>(lvec(0)), rv, (long long)b0 * nc, st);
-  }
-  int rc = solve_root(h, rootA, rv, sizeof(T) == sizeof(double)
-                                        ? reinterpret_cast<double*>(f.lv[0].zv)
-                                        : h->root_vec2 + rc0, nc, st);
+  const int rc = sweep_root<T>(h, f, lvec(0), nc, col0, st);
   if (rc) return rc;
-  if (sizeof(T) != sizeof(double)) {
-    Launch k(h, HSS_K_OTHER, 0.0, st);
-    launch_f64_to_f32(rv, reinterpret_cast<float*>(lvec(0)), (long long)b0 * nc, st);
-  }
   if (lo >= 1) {
     const long long wl = h->wait_budget > 0 ? h->wait_budget : (h->wait_budget < 0 ? 0 : 1LL << 24);
     if (++ln.epoch <= 0) ln.epoch = 1;

@@ -156,8 +156,9 @@ chol64_kernel(double* Mb, int ldm, long long sM, int kb, double* Xb, int ldx, lo
   }
 }
 
-__global__ void copy_rows_kernel(const double* __restrict__ src, int lds, long long ss,
-                                 double* __restrict__ dst, int ldd, long long sd, int r, int nc) {
+template <typename T>
+__global__ void copy_rows_kernel(const T* __restrict__ src, int lds, long long ss,
+                                 T* __restrict__ dst, int ldd, long long sd, int r, int nc) {
   const long long node = blockIdx.x;
   for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < r * nc; e += gridDim.y * blockDim.x) {
     const int i = e % r, j = e / r;
@@ -183,10 +184,16 @@ cudaError_t launch_chol64(double* M, int ldm, long long sM, int kb, double* X, i
   return cudaGetLastError();
 }
 
-cudaError_t launch_copy_rows(const double* src, int lds, long long ss, double* dst, int ldd,
-                             long long sd, int r, int nc, int nodes, cudaStream_t st) {
+template <typename T>
+cudaError_t launch_copy_rows(const T* src, int lds, long long ss, T* dst, int ldd, long long sd,
+                             int r, int nc, int nodes, cudaStream_t st) {
   if (r <= 0 || nc <= 0 || nodes <= 0) return cudaSuccess;
   copy_rows_kernel<<<dim3(nodes, (r * nc + 255) / 256), 256, 0, st>>>(src, lds, ss, dst, ldd, sd,
                                                                      r, nc);
   return cudaGetLastError();
 }
+
+template cudaError_t launch_copy_rows<double>(const double*, int, long long, double*, int, long long,
+                                              int, int, int, cudaStream_t);
+template cudaError_t launch_copy_rows<float>(const float*, int, long long, float*, int, long long, int,
+                                             int, int, cudaStream_t);

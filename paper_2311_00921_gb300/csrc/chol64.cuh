@@ -1,5 +1,5 @@
-// Blocked FP64 Cholesky and triangular solves of a whole tree level as products
-// (chol64.cu holds the kernels; the level routines are below).
+// Blocked FP64 Cholesky, and triangular solves (FP64 and FP32), of a whole tree level
+// as products (chol64.cu and sweep32.cu hold the kernels; the level routines are below).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -7,6 +7,7 @@
 
 #include "../../include/hss.h"
 #include "fxgemm.cuh"
+#include "sweep32.cuh"
 
 // Cholesky factor of the kb x kb block (kb <= 64) at the head of every matrix of a
 // batch, and its inverse: L over the lower triangle of M (ld ldm, stride sM),
@@ -20,8 +21,9 @@ cudaError_t launch_chol64(double* M, int ldm, long long sM, int kb, double* X, i
                           cudaStream_t st);
 
 // dst (r rows per node, ld ldd, stride sd) = src (ld lds, stride ss), nc columns
-cudaError_t launch_copy_rows(const double* src, int lds, long long ss, double* dst, int ldd,
-                             long long sd, int r, int nc, int nodes, cudaStream_t st);
+template <typename T>
+cudaError_t launch_copy_rows(const T* src, int lds, long long ss, T* dst, int ldd, long long sd,
+                             int r, int nc, int nodes, cudaStream_t st);
 
 // Order of the inverted diagonal blocks, and the elements they take per node, for
 // c eliminated columns.  128: a triangular solve of c columns is then c / 128
@@ -34,15 +36,18 @@ inline long long inv_size(int c) {
 }
 
 // One tree level of the factor: n nodes of order b, c columns eliminated.
-struct Level64 {
+template <typename T>
+struct LevelOf {
   int n, b, c;
-  double* M;    // n x b x b, the factored blocks
-  double* Li;   // n x inv_size(c), the inverted diagonal blocks
+  T* M;    // n x b x b, the factored blocks
+  T* Li;   // n x inv_size(c), the inverted diagonal blocks
 
-  Level64 part(int first, int count) const {
+  LevelOf part(int first, int count) const {
     return {count, b, c, M + (long long)first * b * b, Li + (long long)first * inv_size(c)};
   }
 };
+
+using Level64 = LevelOf<double>;
 
 // Where the merge puts a level's Schur complements: the diagonal blocks of the
 // parents PA (ld, stride) for the first `split` nodes, and those of PA2 for the
@@ -63,6 +68,14 @@ inline cudaError_t skinny(int m, int nc, int k, const double* A, int lda, long l
   const FxOperand a{A, lda, sA, ta}, b{B, ldb, sB, true};
   return fx_gemm(m, nc, k, a, b, alpha, Cin ? 1.0 : 0.0, Cin, ldcin, sCin, C, ldc, sC, batch, false,
                  nullptr, 0, 0, st);
+}
+
+inline cudaError_t skinny(int m, int nc, int k, const float* A, int lda, long long sA, bool ta,
+                          const float* B, int ldb, long long sB, float alpha, const float* Cin,
+                          int ldcin, long long sCin, float* C, int ldc, long long sC, int batch,
+                          cudaStream_t st) {
+  return narrow32(m, nc, k, A, lda, sA, ta, B, ldb, sB, alpha, Cin, ldcin, sCin, C, ldc, sC, batch,
+                  st);
 }
 
 #define LV_TRY(kind, flops, call)                                       \
@@ -145,25 +158,25 @@ cudaError_t chol_level64(const Level64& lv, double* P, double* part, int level, 
 // Forward triangular sweep of a level on nc columns: z = L^RR⁻¹ y^R, and
 // y^S - L^SR z to the parent's vector par (r = b - c rows per node; null at the
 // root).  y and z: ld ldy and ldz, b rows per node.  y is overwritten.
-template <typename Log>
-cudaError_t fwd_level64(const Level64& lv, double* y, int ldy, double* z, int ldz, double* par,
-                        int ldpar, int nc, cudaStream_t st, const Log& log) {
+template <typename T, typename Log>
+cudaError_t fwd_level(const LevelOf<T>& lv, T* y, int ldy, T* z, int ldz, T* par, int ldpar,
+                      int nc, cudaStream_t st, const Log& log) {
   const int b = lv.b, c = lv.c, n = lv.n, lb = inv_order(c), r = b - c;
   const long long bb = (long long)b * b, sX = inv_size(c);
   if (c == 0 && par)
-    LV_TRY(HSS_K_OTHER, 0.0, launch_copy_rows(y, ldy, b, par, ldpar, r, r, nc, n, st));
+    LV_TRY(HSS_K_OTHER, 0.0, launch_copy_rows<T>(y, ldy, b, par, ldpar, r, r, nc, n, st));
   for (int k0 = 0; k0 < c; k0 += kInvOrder) {
     const int kb = std::min(kInvOrder, c - k0), rows = b - k0 - kb;
-    const double* X = lv.Li + (long long)(k0 / lb) * lb * lb;
+    const T* X = lv.Li + (long long)(k0 / lb) * lb * lb;
     LV_TRY(HSS_K_TRSV_FWD, (double)kb * kb * nc * n,
-           skinny(kb, nc, kb, X, lb, sX, false, y + k0, ldy, b, 1.0, nullptr, 0, 0, z + k0, ldz, b,
+           skinny(kb, nc, kb, X, lb, sX, false, y + k0, ldy, b, T(1), static_cast<const T*>(nullptr), 0, 0, z + k0, ldz, b,
                   n, st));
     if (rows <= 0) continue;
     const bool last = k0 + kb == c;   // only the S rows are left: the parent's
-    double* yb = y + k0 + kb;
+    T* yb = y + k0 + kb;
     LV_TRY(HSS_K_TRSV_FWD, 2.0 * rows * kb * nc * n,
            skinny(rows, nc, kb, lv.M + (k0 + kb) + (long long)k0 * b, b, bb, false, z + k0, ldz, b,
-                  -1.0, yb, ldy, b, last && par ? par : yb, last && par ? ldpar : ldy,
+                  T(-1), yb, ldy, b, last && par ? par : yb, last && par ? ldpar : ldy,
                   last && par ? r : b, n, st));
   }
   return cudaSuccess;
@@ -171,22 +184,22 @@ cudaError_t fwd_level64(const Level64& lv, double* y, int ldy, double* z, int ld
 
 // Backward sweep: x^S from the parent's vector, x^R = L^RR⁻ᵀ (z - L^SRᵀ x^S),
 // into y; z is overwritten.
-template <typename Log>
-cudaError_t bwd_level64(const Level64& lv, double* y, int ldy, double* z, int ldz,
-                        const double* par, int ldpar, int nc, cudaStream_t st, const Log& log) {
+template <typename T, typename Log>
+cudaError_t bwd_level(const LevelOf<T>& lv, T* y, int ldy, T* z, int ldz, const T* par, int ldpar,
+                      int nc, cudaStream_t st, const Log& log) {
   const int b = lv.b, c = lv.c, n = lv.n, lb = inv_order(c), r = b - c;
   const long long bb = (long long)b * b, sX = inv_size(c);
   if (par && r > 0)
-    LV_TRY(HSS_K_OTHER, 0.0, launch_copy_rows(par, ldpar, r, y + c, ldy, b, r, nc, n, st));
+    LV_TRY(HSS_K_OTHER, 0.0, launch_copy_rows<T>(par, ldpar, r, y + c, ldy, b, r, nc, n, st));
   for (int k0 = c > 0 ? (c - 1) / kInvOrder * kInvOrder : -1; k0 >= 0; k0 -= kInvOrder) {
     const int kb = std::min(kInvOrder, c - k0), rows = b - k0 - kb;
-    const double* X = lv.Li + (long long)(k0 / lb) * lb * lb;
+    const T* X = lv.Li + (long long)(k0 / lb) * lb * lb;
     if (rows > 0)
       LV_TRY(HSS_K_TRSV_BWD, 2.0 * rows * kb * nc * n,
              skinny(kb, nc, rows, lv.M + (k0 + kb) + (long long)k0 * b, b, bb, true, y + k0 + kb,
-                    ldy, b, -1.0, z + k0, ldz, b, z + k0, ldz, b, n, st));
+                    ldy, b, T(-1), z + k0, ldz, b, z + k0, ldz, b, n, st));
     LV_TRY(HSS_K_TRSV_BWD, (double)kb * kb * nc * n,
-           skinny(kb, nc, kb, X, lb, sX, true, z + k0, ldz, b, 1.0, nullptr, 0, 0, y + k0, ldy, b,
+           skinny(kb, nc, kb, X, lb, sX, true, z + k0, ldz, b, T(1), static_cast<const T*>(nullptr), 0, 0, y + k0, ldy, b,
                   n, st));
   }
   return cudaSuccess;
