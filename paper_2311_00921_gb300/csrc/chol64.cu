@@ -160,6 +160,8 @@ template <typename T>
 __global__ void copy_rows_kernel(const T* __restrict__ src, int lds, long long ss,
                                  T* __restrict__ dst, int ldd, long long sd, int r, int nc) {
   const long long node = blockIdx.x;
+  chain_wait();
+  chain_release();
   for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < r * nc; e += gridDim.y * blockDim.x) {
     const int i = e % r, j = e / r;
     dst[node * sd + i + (long long)j * ldd] = src[node * ss + i + (long long)j * lds];
@@ -188,9 +190,8 @@ template <typename T>
 cudaError_t launch_copy_rows(const T* src, int lds, long long ss, T* dst, int ldd, long long sd,
                              int r, int nc, int nodes, cudaStream_t st) {
   if (r <= 0 || nc <= 0 || nodes <= 0) return cudaSuccess;
-  copy_rows_kernel<<<dim3(nodes, (r * nc + 255) / 256), 256, 0, st>>>(src, lds, ss, dst, ldd, sd,
-                                                                     r, nc);
-  return cudaGetLastError();
+  return launch_chained(copy_rows_kernel<T>, dim3(nodes, (r * nc + 255) / 256), 256, 0, st, src, lds,
+                        ss, dst, ldd, sd, r, nc);
 }
 
 template cudaError_t launch_copy_rows<double>(const double*, int, long long, double*, int, long long,

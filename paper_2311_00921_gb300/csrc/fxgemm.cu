@@ -427,6 +427,8 @@ fx_skinny_kernel(const __grid_constant__ FxShape s) {
   double res[NB];
 #pragma unroll
   for (int b = 0; b < NB; ++b) res[b] = 0.0;
+  chain_wait();
+  chain_release();
 
   for (int kt = 0; kt < s.K; kt += kGroup * TEAMS) {
     const int kg = kt + kGroup * team, ke = min(s.K, kg + kGroup), kw = kg + 32 * w;
@@ -578,8 +580,8 @@ cudaError_t launch_skinny(FxShape& s, int batch, cudaStream_t st) {
   const int bytes = skinny_smem<NB, TEAMS>();
   const cudaError_t e = fx_allow_smem(reinterpret_cast<const void*>(kernel), bytes);
   if (e != cudaSuccess) return e;
-  kernel<<<(unsigned)((long long)s.tiles * batch), 128 * TEAMS, bytes, st>>>(s);
-  return cudaGetLastError();
+  return launch_chained(kernel, dim3((unsigned)((long long)s.tiles * batch)), 128 * TEAMS, bytes,
+                        st, s);
 }
 
 template <int BN, bool AKC, bool BKC>

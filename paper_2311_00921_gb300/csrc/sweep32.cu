@@ -47,6 +47,8 @@ narrow32_kernel(const __grid_constant__ Narrow s) {
   for (int h = 0; h < 2; ++h)
 #pragma unroll
     for (int j = 0; j < NC; ++j) acc[h][j] = 0.f;
+  chain_wait();
+  chain_release();
   for (int kc = kChunk * w; kc < s.k; kc += kChunk * kWarps) {
     float a[2][kChunk];
     if (TA) {
@@ -175,12 +177,8 @@ inv32_kernel(const float* __restrict__ Mb, int ldm, long long sM, int c, float* 
 
 template <int NC>
 cudaError_t run_narrow(const Narrow& s, bool ta, int batch, cudaStream_t st) {
-  const unsigned grid = (unsigned)((long long)s.tiles * batch);
-  if (ta)
-    narrow32_kernel<NC, true><<<grid, kThreads, 0, st>>>(s);
-  else
-    narrow32_kernel<NC, false><<<grid, kThreads, 0, st>>>(s);
-  return cudaGetLastError();
+  return launch_chained(ta ? narrow32_kernel<NC, true> : narrow32_kernel<NC, false>,
+                        dim3((unsigned)((long long)s.tiles * batch)), kThreads, 0, st, s);
 }
 
 }  // namespace
