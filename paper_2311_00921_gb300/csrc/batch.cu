@@ -233,7 +233,7 @@ int factor_group(hss_batch_s* bt, Group& g) {
     const int b = t.b;
     const long long br = (long long)b * r;
     const double* Bsrc = (h == 0) ? g.U : t.B;
-    if (ql_blocked<double>(r))
+    if (ql_blocked<double>(b, r, (int)t.nodes))
       TRY(ql_level<double>(Bsrc, t.V, t.T, t.LB, b, r, (int)t.nodes, g.qW, g.q1, g.q2, 0, qs,
                            NoLog()));
     else
@@ -275,7 +275,7 @@ int factor_group(hss_batch_s* bt, Group& g) {
     TRY(cudaStreamWaitEvent(st, g.ev[h], 0));
     const double* Ain = (h == 0) ? g.D : t.A;
     gemm(false, false, b, r, b, 1.0, Ain, b, bb, t.V, b, br, 0.0, g.W, b, br, n, st);
-    if (ql_blocked<double>(r))
+    if (ql_blocked<double>(b, r, (int)t.nodes))
       TRY(ql_tfactor<double>(t.V, t.T, b, r, (int)n, g.tG, g.tP, st, NoLog()));
     gemm(false, false, b, r, r, 1.0, g.W, b, br, t.T, r, rr, 0.0, g.Y, b, br, n, st);
     gemm(true, false, r, r, b, 1.0, t.V, b, br, g.Y, b, br, 0.0, g.X, r, rr, n, st);

@@ -474,7 +474,7 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
       hook.ctx = &bt;
       HSS_TRY(launch_basis_completion<T>(Bsrc, br, P.V, br, P.T_, rr, P.LB, rr, b, r, n, f.bs,
                                          hook, qs));
-    } else if (ql_blocked<T>(r)) {
+    } else if (ql_blocked<T>(b, r, n)) {
       if (sizeof(T) == 8 && !ql_accepts64(b, r)) return HSS_ERR_INVALID_ARG;
       HSS_TRY(ql_level<T>(Bsrc, P.V, P.T_, P.LB, b, r, n, f.bs.X, f.bs.G, f.bs.R1, h->ql_panel, qs,
                           LaunchLog{h, qs, sizeof(T) == 4}));
@@ -535,7 +535,7 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
     }
     if (!tc)
       gemm<T>(h, false, false, b, r, b, T(1), Ain, b, bb, P.V, b, br, T(0), f.W, b, br, n, st);
-    if (ql_blocked<T>(r) && !(h->basis_method == HSS_BASIS_CHOLQR && r <= basis_max_rank<T>()))
+    if (ql_blocked<T>(b, r, n) && !(h->basis_method == HSS_BASIS_CHOLQR && r <= basis_max_rank<T>()))
       HSS_TRY(ql_tfactor<T>(P.V, P.T_, b, r, n, f.bs.R, f.bs.P, st,
                             LaunchLog{h, st, sizeof(T) == 4}));
     gemm<T>(h, false, false, b, r, r, T(1), f.W, b, br, P.T_, r, rr, T(0), f.Y, b, br, n, st);

@@ -31,10 +31,14 @@ cudaError_t launch_ql_tblocks(const T* G, T* Tm, int r, int nodes, cudaStream_t 
 // count up to the SMs: 2.7 -> 1.45 ms; 512 leaves of 512 x 128: 18.9 -> 8.4 ms; 16 of
 // 256 x 32: 0.29 -> 0.24 ms).  In FP32 the one-CTA kernel's products are fast and the
 // launches count: rank 96 loses 2 % of a step, rank 256 gains (leaf 1024: 8.9 ->
-// 3.1 ms, the levels above 2.2 -> 1.3 ms).
+// 3.1 ms, the levels above 2.2 -> 1.3 ms).  At lower ranks it gains on a level with more
+// nodes than SMs and more rows than a CTA has threads, where the one-CTA kernel runs in
+// several waves of two rows a thread (512 leaves of 512 x 128, 3.0 ms of the critical path:
+// the step 22.1 -> 21.0 ms).
 template <typename T>
-bool ql_blocked(int r) {
-  return r > (sizeof(T) == 8 ? 16 : 128);
+bool ql_blocked(int b, int r, int nodes) {
+  if (sizeof(T) == 8) return r > 16;
+  return r > 128 || (r >= 64 && b > 256 && nodes >= 152);
 }
 
 template <typename T>
