@@ -100,7 +100,7 @@ typedef struct {
 } hss_shape;
 
 /* Arithmetic of the refinement residual r = b - A x of the mixed modes.
- * HSS_RESIDUAL_FP64: the HSS matvec in FP64 (the chip's FP64 pipe).
+ * HSS_RESIDUAL_FP64: the HSS matvec in FP64 (exact slicing on the tensor cores).
  * HSS_RESIDUAL_PAIR32: the same matvec with every value held as an unevaluated
  * sum of two FP32 numbers (48-bit significand) and every product and sum done
  * with error-free FP32 transformations on the FP32 pipe; a dot product of
