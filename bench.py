@@ -205,7 +205,7 @@ def traffic_record(kernel, prec):
 
 KERNEL_SOURCES = {"tc_gemm": "tc_gemm_kernel", "tc_syr2k": "tc_gemm_kernel",
                   "gemm": "gemm_tile_kernel", "syr2k": "syr2k_lower_kernel",
-                  "pchol": "pchol_kernel", "ql": "ql_basis_kernel",
+                  "pchol": "chol_panel_kernel", "ql": "ql_basis_kernel",
                   "gemm_skinny": "gemm_n16_kernel", "trsv_fwd": "trsv_fwd_kernel",
                   "trsv_bwd": "trsv_bwd_kernel", "other": "logdet_reduce_kernel",
                   "pair_gemm": "df_gemm_kernel", "basis_gemm": "basis_gemm_kernel",
