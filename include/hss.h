@@ -209,8 +209,9 @@ int hss_logdet(hss_t h, double* out);
 
 /* y = A x with the HSS generators (the product A·b of the construction-error
  * formula in Sec. 5.1): upward pass through U and E, sibling couplings, downward
- * pass, leaf blocks.  FP64.  x and y are device pointers (n x nrhs, ld), must
- * not overlap.  Asynchronous.  Needs no factorization. */
+ * pass, leaf blocks.  FP64: every product within about K 2^-53 of Σ|a||b| in each
+ * component, as a chain of multiply-adds is.  x and y are device pointers (n x nrhs,
+ * ld), must not overlap.  Asynchronous.  Needs no factorization. */
 int hss_matvec(hss_t h, const double* x, double* y, int32_t nrhs, int32_t ld, void* stream);
 
 /* y = A x as hss_matvec, every product and sum in pair-of-FP32 arithmetic

@@ -192,9 +192,10 @@ size_t layout(hss_batch_s* bt, char* base) {
 
 void gemm(bool ta, bool tb, int m, int n, int k, double alpha, const double* A, int lda,
           long long sA, const double* B, int ldb, long long sB, double beta, double* C, int ldc,
-          long long sC, long long batch, cudaStream_t st) {
+          long long sC, long long batch, cudaStream_t st, bool components = true) {
   if (batch > 0)
-    dgemm_batched(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, (int)batch, st);
+    dgemm_batched(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, (int)batch, st,
+                  components);
 }
 
 #define TRY(call)                                                                      \
@@ -274,13 +275,18 @@ int factor_group(hss_batch_s* bt, Group& g) {
     const long long br = (long long)b * r, bb = (long long)b * b, n = t.nodes;
     TRY(cudaStreamWaitEvent(st, g.ev[h], 0));
     const double* Ain = (h == 0) ? g.D : t.A;
-    gemm(false, false, b, r, b, 1.0, Ain, b, bb, t.V, b, br, 0.0, g.W, b, br, n, st);
+    gemm(false, false, b, r, b, 1.0, Ain, b, bb, t.V, b, br, 0.0, g.W, b, br, n, st,
+         false);
     if (ql_blocked<double>(b, r, (int)t.nodes))
       TRY(ql_tfactor<double>(t.V, t.T, b, r, (int)n, g.tG, g.tP, st, NoLog()));
-    gemm(false, false, b, r, r, 1.0, g.W, b, br, t.T, r, rr, 0.0, g.Y, b, br, n, st);
-    gemm(true, false, r, r, b, 1.0, t.V, b, br, g.Y, b, br, 0.0, g.X, r, rr, n, st);
-    gemm(true, false, r, r, r, 1.0, t.T, r, rr, g.X, r, rr, 0.0, g.Z, r, rr, n, st);
-    gemm(false, false, b, r, r, -0.5, t.V, b, br, g.Z, r, rr, 1.0, g.Y, b, br, n, st);
+    gemm(false, false, b, r, r, 1.0, g.W, b, br, t.T, r, rr, 0.0, g.Y, b, br, n, st,
+         false);
+    gemm(true, false, r, r, b, 1.0, t.V, b, br, g.Y, b, br, 0.0, g.X, r, rr, n, st,
+         false);
+    gemm(true, false, r, r, r, 1.0, t.T, r, rr, g.X, r, rr, 0.0, g.Z, r, rr, n, st,
+         false);
+    gemm(false, false, b, r, r, -0.5, t.V, b, br, g.Z, r, rr, 1.0, g.Y, b, br, n, st,
+         false);
     dsyr2k_lower_batched(b, r, Ain, b, bb, g.Y, b, br, t.V, b, br, t.M, b, bb, (int)n, st);
     const Merge64 up{t.split > 0 ? g.ht[h + 1].A : nullptr, 2 * r, 4 * rr, (int)t.split,
                      g.R + (long long)t.mfirst * 4 * rr};

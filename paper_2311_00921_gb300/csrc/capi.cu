@@ -399,12 +399,13 @@ void clear_trace(hss_s* h) {
 template <typename T>
 void gemm(hss_s* h, bool ta, bool tb, int m, int n, int k, T alpha, const T* A, int lda,
           long long sA, const T* B, int ldb, long long sB, T beta, T* C, int ldc, long long sC,
-          int batch, cudaStream_t st) {
+          int batch, cudaStream_t st, bool components = true) {
   if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return;
   Launch l(h, n <= 32 ? HSS_K_GEMM_SKINNY : HSS_K_GEMM, 2.0 * m * n * (double)k * batch, st,
            sizeof(T) == 4);
   if constexpr (std::is_same<T, double>::value)
-    dgemm_batched(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, st);
+    dgemm_batched(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, st,
+                  components);
   else
     gemm_batched<T>(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, st);
 }
@@ -534,14 +535,19 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
       }
     }
     if (!tc)
-      gemm<T>(h, false, false, b, r, b, T(1), Ain, b, bb, P.V, b, br, T(0), f.W, b, br, n, st);
+      gemm<T>(h, false, false, b, r, b, T(1), Ain, b, bb, P.V, b, br, T(0), f.W, b, br, n, st,
+            false);
     if (ql_blocked<T>(b, r, n) && !(h->basis_method == HSS_BASIS_CHOLQR && r <= basis_max_rank<T>()))
       HSS_TRY(ql_tfactor<T>(P.V, P.T_, b, r, n, f.bs.R, f.bs.P, st,
                             LaunchLog{h, st, sizeof(T) == 4}));
-    gemm<T>(h, false, false, b, r, r, T(1), f.W, b, br, P.T_, r, rr, T(0), f.Y, b, br, n, st);
-    gemm<T>(h, true, false, r, r, b, T(1), P.V, b, br, f.Y, b, br, T(0), f.X, r, rr, n, st);
-    gemm<T>(h, true, false, r, r, r, T(1), P.T_, r, rr, f.X, r, rr, T(0), f.Z, r, rr, n, st);
-    gemm<T>(h, false, false, b, r, r, T(-0.5), P.V, b, br, f.Z, r, rr, T(1), f.Y, b, br, n, st);
+    gemm<T>(h, false, false, b, r, r, T(1), f.W, b, br, P.T_, r, rr, T(0), f.Y, b, br, n, st,
+            false);
+    gemm<T>(h, true, false, r, r, b, T(1), P.V, b, br, f.Y, b, br, T(0), f.X, r, rr, n, st,
+            false);
+    gemm<T>(h, true, false, r, r, r, T(1), P.T_, r, rr, f.X, r, rr, T(0), f.Z, r, rr, n, st,
+            false);
+    gemm<T>(h, false, false, b, r, r, T(-0.5), P.V, b, br, f.Z, r, rr, T(1), f.Y, b, br, n, st,
+            false);
     if (tc) {
       if constexpr (std::is_same<T, float>::value) {
         Launch k(h, HSS_K_TC_SYR2K, 2.0 * r * b * (b + 1.0) * n, st);

@@ -12,15 +12,27 @@
 // of at most 2^24, so every MMA is exact.  At the end of a group the eight
 // accumulators are put together as two integers and added to the FP64 result.
 //
-// Error of one group: cutting each operand at 2^-63 of its row's largest
-// element, and the dropped digit products, about 2^-63 of max|a| max|b| a product:
-// far below the 2^-53 of a partial sum that each step of a DFMA chain rounds
-// off, also where a row's largest element dwarfs the others (seven digits, whose
-// error is 2^-56 of max|a| max|b|, are not enough there: the solves of kernel
-// matrices lost a factor of three to five against the DFMA chain).  Rows with an
-// element that is not finite or whose largest magnitude is outside
-// [2^-470, 2^470] take a DFMA loop instead, so that infinities, NaN and
-// overflow behave as in the plain product.
+// Error of one group: cutting each operand at 2^-63 of its row's scale (at most twice
+// its largest element), and the dropped digit products, together at most 2^-60.5 of
+// the scales' product per inner index (2^-64 √K in the mean over random digits).  That
+// is relative to the rows' largest elements; a DFMA chain is within K 2^-53 of Σ|a||b|,
+// far less where the large elements of one row meet zeros or small elements of the
+// other.  So each element's S = Σ|a||b| is accumulated beside its digits' products, by a
+// 37th MMA on the two leading digits' absolute values (FP16 accumulators: S above
+// 65504 is as good as infinite).  Where S is below 2^-8 of the scales' product, the
+// group's part of that element is summed by DFMA; elsewhere the error is at most
+// K 2^-52.5 of Σ|a||b|, 2^-56 √K in the mean.  The products of the Householder
+// transformations, whose error in any arithmetic is relative to the norms of rows and
+// columns (a chain's bound K 2^-53 of them is 2^5 of the above), do without S
+// (components = false): the reflectors' unit entries and zeros would send up to 22 % of
+// their elements to the DFMA pipe.  Batch of ten: 11.4 ms without S, 13.9 ms with S
+// in all products, 12.0 ms so; D x of 512 leaves and 16 columns is 5 % slower with S.
+// (Seven digits, whose error is 2^-56 of max|a| max|b|, are not enough: the solves of
+// kernel matrices lost a factor of three to five against the DFMA chain.)
+//
+// Rows with an element that is not finite or whose largest magnitude is outside
+// [2^-470, 2^470] take a DFMA loop as a whole, so that infinities, NaN, overflow and
+// denormals behave as in the plain product.
 //
 // Layout: a CTA has 4 warps and a 64 x BN tile of C (BN = 32, 16 or 8 columns;
 // a warp 16 rows and every column).  Per group the operands' strips are read
@@ -47,6 +59,8 @@ constexpr int kGroup = 128;     // inner indices with one scale
 constexpr int kDigits = 8;
 constexpr int kPitch = 2 * kChunk + 16;   // bytes of a row of digits in shared memory
 constexpr int kHiBig = (1023 + 470) << 20, kHiSmall = (1023 - 470) << 20;
+constexpr int kZeroRow = 1 << 16;   // exponent of a row of zeros: shifts every digit out
+constexpr float kLeast = 64.f;      // 2^-8 of the scales' product, in the unit of S (128 a scale)
 
 struct FxShape {
   int m, n, K, K1;   // K1: inner indices of each part, K in all
@@ -63,6 +77,7 @@ struct FxShape {
   int ldpa;
   long long sPA;
   int tiles_m, tiles_n, tiles;
+  int components;
 };
 
 HSS_DEVINL uint32_t smem_of(const void* p) {
@@ -128,6 +143,42 @@ HSS_DEVINL void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// S += |a| |b| in FP16, of the operands' absolute leading parts
+HSS_DEVINL void mma_abs(uint32_t (&c)[2], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f16.f16.f16.f16 {%0, %1}, {%2, %3, %4, %5}, {%6, %7}, "
+      "{%0, %1};"
+      : "+r"(c[0]), "+r"(c[1])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// |d0 + d1 / 256|, two digits of a pair of elements (digit units of the first)
+HSS_DEVINL uint32_t leading(uint32_t d0, uint32_t d1) {
+  uint32_t r;
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(d1), "r"(0x1c001c00u), "r"(d0));
+  return r & 0x7fff7fffu;
+}
+
+// half h of an fp16x2
+HSS_DEVINL float half_of(uint32_t v, int h) {
+  float f;
+  asm("{.reg .b16 t; cvt.u16.u32 t, %1; cvt.f32.f16 %0, t;}" : "=f"(f) : "r"(h ? v >> 16 : v));
+  return f;
+}
+
+// magnitude of v for the row maxima: its high word, not zero if v is not
+HSS_DEVINL int magnitude(double v) {
+  return (__double2hiint(v) & 0x7fffffff) | (__double2loint(v) != 0);
+}
+
+// biased exponent (+ 1) of a row's scale from its largest magnitude: |v| < 0.996 2^(E - 1022),
+// a mantissa near 2 goes up to the next power, so that the digits' range holds it;
+// odd: the row is outside the sliced range
+HSS_DEVINL int row_exponent(int h, int& odd) {
+  odd |= h >= kHiBig || (h > 0 && h < kHiSmall);
+  return h ? ((h + 0x2100) >> 20) + 1 : kZeroRow;
+}
+
 // R rows (from row0 on) of one operand's part (contiguous inner indices 0 .. K-1
 // of one array).  Rows past the last are read as copies of it: their results are
 // not stored.
@@ -142,7 +193,7 @@ struct Strip {
   }
   HSS_DEVINL double at(int r, int k) const { return row(r)[KC ? (long long)k : (long long)k * ld]; }
 
-  // mx[r] = largest high word (sign removed) of row r over [k0, k1); mx is cleared
+  // mx[r] = largest magnitude() of row r over [k0, k1); mx is cleared
   HSS_DEVINL void maxima(int k0, int k1, int* mx) const {
     const int tid = threadIdx.x;
     if (KC) {
@@ -155,13 +206,13 @@ struct Strip {
           const double* q = row(r + 4 * u) + k0 + lane;
 #pragma unroll
           for (int j = 0; j < kGroup / 32; ++j)
-            v[u][j] = k0 + lane + 32 * j < k1 ? __double2hiint(q[32 * j]) : 0;
+            v[u][j] = k0 + lane + 32 * j < k1 ? magnitude(q[32 * j]) : 0;
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           int h = 0;
 #pragma unroll
-          for (int j = 0; j < kGroup / 32; ++j) h = max(h, v[u][j] & 0x7fffffff);
+          for (int j = 0; j < kGroup / 32; ++j) h = max(h, v[u][j]);
           h = __reduce_max_sync(0xffffffffu, h);
           if (lane == 0) mx[r + 4 * u] = h;
         }
@@ -175,12 +226,12 @@ struct Strip {
       for (; k + 15 * S < n; k += 16 * S) {
         int v[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j, q += step) v[j] = __double2hiint(*q);
+        for (int j = 0; j < 16; ++j, q += step) v[j] = magnitude(*q);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) h = max(h, v[j] & 0x7fffffff);
+        for (int j = 0; j < 16; ++j) h = max(h, v[j]);
       }
 #pragma unroll 4
-      for (; k < n; k += S, q += step) h = max(h, __double2hiint(*q) & 0x7fffffff);
+      for (; k < n; k += S, q += step) h = max(h, magnitude(*q));
       atomicMax(mx + r, h);
     }
   }
@@ -231,6 +282,83 @@ struct Strip {
     }
   }
 };
+
+// res += Σ_k A B over [k0, k1) by a DFMA chain, for the elements set in `which`
+// (bit 4 b + e: fragment register e of column block b)
+template <int NB, typename SA, typename SB>
+HSS_DEVINL void plain_group(const SA& A, const SB& B, int k0, int k1, uint32_t which,
+                            double (&res)[NB][4]) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int k = k0; k < k1; ++k)
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int r = w * 16 + (lane >> 2) + 8 * (e >> 1);
+        const int c = 8 * b + 2 * (lane & 3) + (e & 1);
+        if (which >> (4 * b + e) & 1) res[b][e] = fma(A.at(r, k), B.at(c, k), res[b][e]);
+      }
+}
+
+// Σ_k a(l, k) b(l, k) over [k0, k1) for the lanes l set in `bad`, by the warp together; the
+// lane's own sum is returned.  A warp-wide FP64 instruction takes 64 clocks of its SM
+// quarter: four sums at a time on eight lanes each cost 300 clocks a sum, one on 32
+// lanes 600, a lane's own chain 8192.
+template <typename At, typename Bt>
+HSS_DEVINL double warp_dots(uint32_t bad, int k0, int k1, At a, Bt b) {
+  const int lane = threadIdx.x & 31;
+  double mine = 0.0;
+  while (bad) {
+    const bool four = __popc(bad) > 2;
+    const int width = four ? 8 : 32;
+    int src[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      src[q] = __ffs(bad) - 1;   // -1: none left
+      if (q == 0 || four) bad &= bad - 1;
+    }
+    int l = src[0];
+#pragma unroll
+    for (int q = 1; q < 4; ++q)
+      if (four && lane >> 3 == q && src[q] >= 0) l = src[q];
+    double v = 0.0;
+#pragma unroll 4
+    for (int k = k0 + (lane & (width - 1)); k < k1; k += width) v = fma(a(l, k), b(l, k), v);
+    if (!four) {
+      v += __shfl_xor_sync(0xffffffffu, v, 16);
+      v += __shfl_xor_sync(0xffffffffu, v, 8);
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double x = __shfl_sync(0xffffffffu, v, 8 * q);
+      if (lane == src[q] && (q == 0 || four)) mine = x;
+    }
+  }
+  return mine;
+}
+
+// plain_group's sums by the warp together where they are few.  Called by whole warps.
+template <int NB, typename SA, typename SB>
+__device__ __noinline__ void small_sums(const SA& A, const SB& B, int k0, int k1, uint32_t which,
+                                        double (&res)[NB][4]) {
+  const int w = threadIdx.x >> 5;
+  if (__reduce_add_sync(0xffffffffu, __popc(which)) > 64 * NB) {
+    plain_group<NB>(A, B, k0, k1, which, res);
+    return;
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const uint32_t bad = __ballot_sync(0xffffffffu, which >> (4 * b + e) & 1);
+      if (!bad) continue;
+      res[b][e] += warp_dots(
+          bad, k0, k1, [&](int l, int k) { return A.at(w * 16 + (l >> 2) + 8 * (e >> 1), k); },
+          [&](int l, int k) { return B.at(8 * b + 2 * (l & 3) + (e & 1), k); });
+    }
+}
 
 template <int BN>
 constexpr int fx_smem() {
@@ -283,26 +411,15 @@ fx_gemm_kernel(const __grid_constant__ FxShape s) {
     B.maxima(kg, ke, ex + kRows);
     __syncthreads();
     int odd = 0;
-    for (int r = tid; r < kRows + BN; r += kThreads) {
-      const int h = ex[r];
-      odd |= h >= kHiBig || (h > 0 && h < kHiSmall);
-      // |v| < 0.996 2^(E - 1022): a mantissa near 2 goes up to the next power,
-      // so that the digits' range holds it
-      ex[r] = (h ? (h + 0x2100) >> 20 : 1023) + 1;
-    }
+    for (int r = tid; r < kRows + BN; r += kThreads) ex[r] = row_exponent(ex[r], odd);
     if (__syncthreads_or(odd)) {   // plain FP64 for this group
-      for (int k = kg; k < ke; ++k)
-#pragma unroll
-        for (int b = 0; b < NB; ++b)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int r = w * 16 + (lane >> 2) + 8 * (e >> 1);
-            const int c = 8 * b + 2 * (lane & 3) + (e & 1);
-            res[b][e] = fma(A.at(r, k), B.at(c, k), res[b][e]);
-          }
+      plain_group<NB>(A, B, kg, ke, 0xffffffffu, res);
       __syncthreads();
       continue;
     }
+    uint32_t abs_sum[NB][2];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) abs_sum[b][0] = abs_sum[b][1] = 0;
 #pragma unroll
     for (int q = 0; q < kDigits; ++q)
 #pragma unroll
@@ -326,25 +443,42 @@ fx_gemm_kernel(const __grid_constant__ FxShape s) {
             smem_of(smA) + (w * 16 + (lane & 15)) * kPitch + ks * 32 + (lane >> 4) * 16;
 #pragma unroll
         for (int q = 0; q < kDigits; ++q) ldmatrix4(a[q], aa + q * kRows * kPitch);
+        uint32_t la[4];
+        if (s.components) {
+#pragma unroll
+          for (int p = 0; p < 4; ++p) la[p] = leading(a[0][p], a[1][p]);
+        }
         // two blocks of 8 columns per load (BN = 8: both halves of the 16 indices of one)
         const uint32_t ba = smem_of(smB) + ks * 32 + ((lane >> 3) & 1) * 16 +
                             ((lane & 7) + (NB > 1 ? (lane >> 4) << 3 : 0)) * kPitch;
 #pragma unroll
-        for (int b = 0; b < NB; b += 2)
+        for (int b = 0; b < NB; b += 2) {
+          uint32_t v0[4];
 #pragma unroll
           for (int j = 0; j < kDigits; ++j) {
             uint32_t v[4];
             ldmatrix4(v, ba + (j * BN + 8 * b) * kPitch);
+            if (j == 0) {
+#pragma unroll
+              for (int p = 0; p < 4; ++p) v0[p] = v[p];
+            }
+            if (j == 1 && s.components) {
+              mma_abs(abs_sum[b], la, leading(v0[0], v[0]), leading(v0[1], v[1]));
+              if (NB > 1)
+                mma_abs(abs_sum[b + (NB > 1)], la, leading(v0[2], v[2]), leading(v0[3], v[3]));
+            }
 #pragma unroll
             for (int i = 0; i + j < kDigits; ++i) {
               mma_f16(acc[i + j][b], a[i], v[0], v[1]);
               if (NB > 1) mma_f16(acc[i + j][b + (NB > 1)], a[i], v[2], v[3]);
             }
           }
+        }
       }
       __syncthreads();
     }
-    // the group's sum: 2^(ea + eb - 70) (H 2^32 + L)
+    // the group's sum: 2^(ea + eb - 70) (H 2^32 + L); by DFMA where S is small
+    uint32_t small = 0;
 #pragma unroll
     for (int b = 0; b < NB; ++b)
 #pragma unroll
@@ -357,9 +491,17 @@ fx_gemm_kernel(const __grid_constant__ FxShape s) {
         }
         const int r = w * 16 + (lane >> 2) + 8 * (e >> 1);
         const int c = 8 * b + 2 * (lane & 3) + (e & 1);
-        const double scale = __hiloint2double((ex[r] + ex[kRows + c] - 1093) << 20, 0);
+        const int E = ex[r] + ex[kRows + c];
+        if (E >= kZeroRow) continue;
+        if (s.components && half_of(abs_sum[b][e >> 1], e & 1) < kLeast) {
+          // not for results that are not stored
+          if (i0 + r < s.m && j0 + c < s.n) small |= 1u << (4 * b + e);
+          continue;
+        }
+        const double scale = __hiloint2double((E - 1093) << 20, 0);
         res[b][e] = fma(fma((double)H, 4294967296.0, (double)L), scale, res[b][e]);
       }
+    if (__any_sync(0xffffffffu, small)) small_sums<NB>(A, B, kg, ke, small, res);
     __syncthreads();
   }
   }
@@ -398,14 +540,15 @@ fx_gemm_kernel(const __grid_constant__ FxShape s) {
 // reads the strips twice and passes them through shared memory, takes 24.7 us.
 template <int NB, int TEAMS>
 constexpr int skinny_smem() {
-  return TEAMS * 4 * (4 * NB) * 2 * 32 * (int)sizeof(float4);
+  return TEAMS * 4 * NB * (4 * 2 * 32 * (int)sizeof(float4) + 2 * 32 * (int)sizeof(uint32_t));
 }
 
 template <int NB, int TEAMS, bool AKC>
 __global__ void __launch_bounds__(128 * TEAMS, (NB == 1 ? 4 : 2) / TEAMS)
 fx_skinny_kernel(const __grid_constant__ FxShape s) {
   constexpr int R = 16, BN = 8 * NB, E = 4 * NB;   // E: fragment registers
-  extern __shared__ __align__(16) float4 xch[];    // [team][warp][E][2][lane]
+  extern __shared__ __align__(16) float4 xch[];    // [team][warp][E][2][lane], then the
+  uint32_t* xsum = reinterpret_cast<uint32_t*>(xch + TEAMS * 4 * E * 64);   // S's [..][NB][2][lane]
   __shared__ int mx[TEAMS][4][R + BN];
   const int tid = threadIdx.x, lane = tid & 31, w = (tid >> 5) & 3, team = tid >> 7;
   const int g = lane >> 2, t = lane & 3;
@@ -449,7 +592,7 @@ fx_skinny_kernel(const __grid_constant__ FxShape s) {
 #pragma unroll
       for (int q = 0; q < 2; ++q)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) x = max(x, __double2hiint(v[q][j]) & 0x7fffffff);
+        for (int j = 0; j < 4; ++j) x = max(x, magnitude(v[q][j]));
       x = max(x, __shfl_xor_sync(0xffffffffu, x, 1));
       return max(x, __shfl_xor_sync(0xffffffffu, x, 2));
     };
@@ -465,10 +608,9 @@ fx_skinny_kernel(const __grid_constant__ FxShape s) {
     }
     __syncthreads();
     int odd = 0;
-    auto exponent = [&](int r) {   // as in fx_gemm_kernel
-      const int h = max(max(mx[team][0][r], mx[team][1][r]), max(mx[team][2][r], mx[team][3][r]));
-      odd |= h >= kHiBig || (h > 0 && h < kHiSmall);
-      return (h ? (h + 0x2100) >> 20 : 1023) + 1;
+    auto exponent = [&](int r) {
+      return row_exponent(
+          max(max(mx[team][0][r], mx[team][1][r]), max(mx[team][2][r], mx[team][3][r])), odd);
     };
     int ea[2], eb[NB];
 #pragma unroll
@@ -483,6 +625,9 @@ fx_skinny_kernel(const __grid_constant__ FxShape s) {
       for (int b = 0; b < NB; ++b)
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[d][b][e] = 0.f;
+    uint32_t abs_sum[NB][2];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) abs_sum[b][0] = abs_sum[b][1] = 0;
     if (!plain) {
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
@@ -498,6 +643,15 @@ fx_skinny_kernel(const __grid_constant__ FxShape s) {
           for (int p = 0; p < 4; ++p)   // fragment register p: row half p & 1, indices p >> 1
             digits(fixed_point(av[p & 1][q][2 * (p >> 1)], ea[p & 1]),
                    fixed_point(av[p & 1][q][2 * (p >> 1) + 1], ea[p & 1]), ad[p]);
+          if (s.components) {
+            uint32_t la[4];
+#pragma unroll
+            for (int p = 0; p < 4; ++p) la[p] = leading(ad[p][0], ad[p][1]);
+#pragma unroll
+            for (int b = 0; b < NB; ++b)
+              mma_abs(abs_sum[b], la, leading(bd[b][0][0], bd[b][0][1]),
+                      leading(bd[b][1][0], bd[b][1][1]));
+          }
 #pragma unroll
           for (int i = 0; i < kDigits; ++i) {
             const uint32_t a[4] = {ad[0][i], ad[1][i], ad[2][i], ad[3][i]};
@@ -518,13 +672,35 @@ fx_skinny_kernel(const __grid_constant__ FxShape s) {
         for (int h = 0; h < 2; ++h)
           mine[((b * 4 + e) * 2 + h) * 32] = make_float4(acc[4 * h][b][e], acc[4 * h + 1][b][e],
                                                          acc[4 * h + 2][b][e], acc[4 * h + 3][b][e]);
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        xsum[((team * 4 + w) * NB + b) * 64 + h * 32 + lane] = abs_sum[b][h];
     __syncthreads();
     // warp w: fragment register w of every block, row g + 8 (w >> 1), column 2 t + (w & 1)
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
       const int ex =
           __shfl_sync(0xffffffffu, eb[b], (2 * t + (w & 1)) * 4) + (w & 2 ? ea[1] : ea[0]);
+      const int row = 8 * (w >> 1) + g, col = 8 * b + 2 * t + (w & 1);
       if (!plain) {
+        float sum = 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          sum += half_of(xsum[((team * 4 + u) * NB + b) * 64 + (w >> 1) * 32 + lane], w & 1);
+        const bool zero = ex >= kZeroRow, small = s.components && !zero && sum < kLeast;
+        // by DFMA; not for results that are not stored
+        const uint32_t bad = __ballot_sync(0xffffffffu, small && i0 + row < s.m && col < s.n);
+        if (bad)
+          res[b] += warp_dots(
+              bad, kg, ke,
+              [&](int l, int k) {
+                const long long i = i0 + 8 * (w >> 1) + (l >> 2);
+                return A[AKC ? i * lda + k : i + k * lda];
+              },
+              [&](int l, int k) { return B[(8 * b + 2 * (l & 3) + (w & 1)) * ldb + k]; });
+        if (zero || small) continue;
         long long v[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -541,8 +717,7 @@ fx_skinny_kernel(const __grid_constant__ FxShape s) {
         const double scale = __hiloint2double((ex - 1093) << 20, 0);
         res[b] = fma(fma((double)v[0], 4294967296.0, (double)v[1]), scale, res[b]);
       } else {   // plain FP64 for this group
-        const int i = min(i0 + 8 * (w >> 1) + g, s.m - 1);
-        const int j = min(8 * b + 2 * t + (w & 1), s.n - 1);
+        const int i = min(i0 + row, s.m - 1), j = min(col, s.n - 1);
         for (int k = kg; k < ke; ++k)
           res[b] = fma(A[AKC ? i * lda + k : i + k * lda], B[j * ldb + k], res[b]);
       }
@@ -630,9 +805,9 @@ cudaError_t fx_allow_smem(const void* kernel, int bytes) {
 cudaError_t fx_gemm(int m, int n, int K, const FxOperand& a, const FxOperand& b, double alpha,
                     double beta, const double* Cin, int ldcin, long long sCin, double* C, int ldc,
                     long long sC, int batch, bool lower, double* PA, int ldpa, long long sPA,
-                    cudaStream_t st) {
+                    cudaStream_t st, bool components) {
   FxShape s{m, n, K, a.p2 ? K / 2 : K, a, b, alpha, beta, Cin ? Cin : C, ldcin, sCin, C, ldc, sC, lower ? 1 : 0,
-            PA, ldpa, sPA, 0, 0, 0};
+            PA, ldpa, sPA, 0, 0, 0, components ? 1 : 0};
   // Narrow products (B's inner index contiguous).  Up to 8 columns fx_skinny_kernel is
   // the faster one at every size (512 x 512, 512 nodes: 481 against 506 us; 128 nodes:
   // 128 against 150; 128 x 128, 8 nodes: 6.2 against 10.5).  With 9 to 16 it wins while
@@ -655,7 +830,7 @@ cudaError_t fx_gemm(int m, int n, int K, const FxOperand& a, const FxOperand& b,
 
 void dgemm_batched(bool transA, bool transB, int m, int n, int k, double alpha, const double* A,
                    int lda, long long sA, const double* B, int ldb, long long sB, double beta,
-                   double* C, int ldc, long long sC, int batch, cudaStream_t st) {
+                   double* C, int ldc, long long sC, int batch, cudaStream_t st, bool components) {
   if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return;
   // A few inner indices and columns on few rows (the tree of a rank <= 8 matrix):
   // the FP64 pipe's kernels take 4.2 us against 6.2 us, whose digits are padded to
@@ -668,16 +843,18 @@ void dgemm_batched(bool transA, bool transB, int m, int n, int k, double alpha, 
     return;
   }
   const FxOperand a{A, lda, sA, transA}, b{B, ldb, sB, !transB};
-  fx_gemm(m, n, k, a, b, alpha, beta, C, ldc, sC, C, ldc, sC, batch, false, nullptr, 0, 0, st);
+  fx_gemm(m, n, k, a, b, alpha, beta, C, ldc, sC, C, ldc, sC, batch, false, nullptr, 0, 0, st,
+          components);
 }
 
 void dsyr2k_lower_batched(int m, int k, const double* A, int lda, long long sA, const double* P,
                           int ldp, long long sP, const double* Q, int ldq, long long sQ, double* M,
                           int ldm, long long sM, int batch, cudaStream_t st) {
   if (m <= 0 || k <= 0 || batch <= 0) return;
-  // A - [P Q] [Q P]ᵀ
+  // A - [P Q] [Q P]ᵀ, a Householder transformation
   const FxOperand a{P, ldp, sP, false, Q, ldq, sQ}, b{Q, ldq, sQ, false, P, ldp, sP};
-  fx_gemm(m, m, 2 * k, a, b, -1.0, 1.0, A, lda, sA, M, ldm, sM, batch, true, nullptr, 0, 0, st);
+  fx_gemm(m, m, 2 * k, a, b, -1.0, 1.0, A, lda, sA, M, ldm, sM, batch, true, nullptr, 0, 0, st,
+          /*components=*/false);
 }
 
 void dsyrk_lower_batched(int m, int k, const double* A, int lda, long long sA, const double* P,

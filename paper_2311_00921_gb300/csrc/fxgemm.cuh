@@ -18,11 +18,14 @@ struct FxOperand {
 // C (m x n) = alpha a bᵀ + beta Cin for `batch` problems, a m x K and b n x K.
 // lower: only elements on and below the diagonal (m = n).  PA (may be null):
 // node z's result also goes, both triangles, to the diagonal block at offset
-// (z & 1) m of parent block z / 2.  Cin may be C.
+// (z & 1) m of parent block z / 2.  Cin may be C.  components: every element
+// within about the bound of a DFMA chain, K 2^-53 Σ|a||b|; else (Householder
+// transformations) within K 2^-58.5 of the largest |a| times the largest |b| of its row
+// and column in each 128 inner indices.
 cudaError_t fx_gemm(int m, int n, int K, const FxOperand& a, const FxOperand& b, double alpha,
                     double beta, const double* Cin, int ldcin, long long sCin, double* C, int ldc,
                     long long sC, int batch, bool lower, double* PA, int ldpa, long long sPA,
-                    cudaStream_t st);
+                    cudaStream_t st, bool components = true);
 
 // opts a kernel into `bytes` of dynamic shared memory, once per device and kernel
 cudaError_t fx_allow_smem(const void* kernel, int bytes);
@@ -33,7 +36,8 @@ cudaError_t fx_allow_smem(const void* kernel, int bytes);
 // in fxgemm.cu leaves them on the FP64 pipe.
 void dgemm_batched(bool transA, bool transB, int m, int n, int k, double alpha, const double* A,
                    int lda, long long sA, const double* B, int ldb, long long sB, double beta,
-                   double* C, int ldc, long long sC, int batch, cudaStream_t st);
+                   double* C, int ldc, long long sC, int batch, cudaStream_t st,
+                   bool components = true);
 void dsyr2k_lower_batched(int m, int k, const double* A, int lda, long long sA, const double* P,
                           int ldp, long long sP, const double* Q, int ldq, long long sQ, double* M,
                           int ldm, long long sM, int batch, cudaStream_t st);

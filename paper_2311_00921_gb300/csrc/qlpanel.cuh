@@ -46,7 +46,8 @@ void level_gemm(bool ta, bool tb, int m, int n, int k, T alpha, const T* A, int 
                 const T* B, int ldb, long long sB, T beta, T* C, int ldc, long long sC, int batch,
                 cudaStream_t st) {
   if constexpr (std::is_same<T, double>::value)
-    dgemm_batched(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, st);
+    dgemm_batched(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, st,
+                  /*components=*/false);
   else
     gemm_batched<T>(ta, tb, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, st);
 }
@@ -105,7 +106,7 @@ cudaError_t ql_tfactor(const T* V, T* Tm, int b, int r, int n, T* G, T* P, cudaS
     if constexpr (std::is_same<T, double>::value) {
       const FxOperand v{V, b, br, true};
       fx_gemm(r, r, b, v, v, 1.0, 0.0, nullptr, 0, 0, G, r, rr, n, /*lower=*/true, nullptr, 0, 0,
-              st);
+              st, /*components=*/false);
     } else {
       level_gemm<T>(true, false, r, r, b, T(1), V, b, br, V, b, br, T(0), G, r, rr, n, st);
     }
