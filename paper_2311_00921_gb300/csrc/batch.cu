@@ -41,7 +41,9 @@ struct Height {
   double *E = nullptr, *S = nullptr, *yv = nullptr, *ldp = nullptr;
   double *Li = nullptr, *zv = nullptr;   // inverted diagonal blocks, forward sweep's z (chol64.cuh)
 
-  Level64 level() const { return {(int)nodes, b, c, M, Li}; }
+  int* Fl = nullptr;                     // which blocks are used without a correction
+
+  Level64 level() const { return {(int)nodes, b, c, M, Li, Fl}; }
 };
 
 struct Group {
@@ -56,6 +58,7 @@ struct Group {
   double *qW = nullptr, *q1 = nullptr, *q2 = nullptr;   // basis chain's scratch (qlpanel.cuh)
   double *tG = nullptr, *tP = nullptr, *cP = nullptr;   // main chain's: T factor, Cholesky rows
   double *rootLi = nullptr, *rootz = nullptr;
+  int* rootFl = nullptr;
   long long rows = 0;          // leaf-level rows of the group
   std::vector<long long> row_off;   // member -> row offset in xg
   cudaStream_t st = nullptr, qs = nullptr;
@@ -140,6 +143,7 @@ size_t layout(hss_batch_s* bt, char* base) {
       }
       t.S = bp.take<double>((t.nodes / 2) * rr);
       t.Li = bp.take<double>(t.nodes * inv_size(t.c));
+      t.Fl = bp.take<int>(t.nodes * flag_size(t.c));
       t.zv = bp.take<double>(t.nodes * t.b * kCols);
       ldp_total += t.nodes;
     }
@@ -151,6 +155,7 @@ size_t layout(hss_batch_s* bt, char* base) {
     g.rootvec = bp.take<double>((size_t)nm * 2 * r * kCols);
     g.rootz = bp.take<double>((size_t)nm * 2 * r * kCols);
     g.rootLi = bp.take<double>((size_t)nm * inv_size(2 * r));
+    g.rootFl = bp.take<int>((size_t)nm * flag_size(2 * r));
     g.W = bp.take<double>(n0 * leaf * r);
     g.Y = bp.take<double>(n0 * leaf * r);
     g.X = bp.take<double>(n0 * rr);
@@ -214,7 +219,7 @@ struct NoLog {
 };
 
 Level64 root_level(const Group& g) {
-  return {(int)g.member.size(), 2 * g.r, 2 * g.r, g.R, g.rootLi};
+  return {(int)g.member.size(), 2 * g.r, 2 * g.r, g.R, g.rootLi, g.rootFl};
 }
 
 // Basis completion, Cholesky and sweeps run as in the single path (qlpanel.cuh,

@@ -50,6 +50,7 @@ struct LevelT {
   T* B = nullptr;   // n x b x r bases fed to the QL (levels 1 .. L-1)
   T* yv = nullptr;  // level vector of the solve: (n b) x kSolveCols
   T* Li = nullptr;  // inverted diagonal blocks of L^RR (chol64.cuh)
+  int* Fl = nullptr;  // FP64: which of them are used without a correction
   T* zv = nullptr;  // the forward sweep's z^R, laid out as yv
 };
 
@@ -200,6 +201,7 @@ void layout_factor(Bump& bp, Factor<T>& f, int L, int leaf, int r) {
       P.Li = bp.take<T>((size_t)P.n * inv_size(P.c));
       P.zv = bp.take<T>((size_t)P.n * P.b * kSolveCols);
     }
+    if (sizeof(T) == 8) P.Fl = bp.take<int>((size_t)P.n * flag_size(P.c));
   }
   if (sizeof(T) == 8) f.P = bp.take<T>(nL * std::max(leaf, 2) * 64);
   f.W = bp.take<T>(nL * leaf * r);
@@ -564,7 +566,7 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
     if (c == 0 && cudaMemsetAsync(slots, 0, sizeof(double) * n, st) != cudaSuccess)
       return HSS_ERR_CUDA;
     if constexpr (std::is_same<T, double>::value) {
-      HSS_TRY(chol_level64({n, b, c, P.M, P.Li}, f.P, slots, l, 0, h->status, {Q.A, ldq, sq, n},
+      HSS_TRY(chol_level64({n, b, c, P.M, P.Li, P.Fl}, f.P, slots, l, 0, h->status, {Q.A, ldq, sq, n},
                            st, LaunchLog{h, st}));
     } else {
       // FP32: per panel of kPanel columns a per-node panel kernel (diagonal block
@@ -619,7 +621,7 @@ int factor_levels(hss_s* h, Factor<T>& f, T* zq, cudaStream_t st, bool split_d) 
 
 // the FP64 root block R as a level of one node with every column eliminated
 Level64 root_level(hss_s* h, double* R) {
-  return {1, 2 * h->rank, 2 * h->rank, R, h->f64.lv[0].Li};
+  return {1, 2 * h->rank, 2 * h->rank, R, h->f64.lv[0].Li, h->f64.lv[0].Fl};
 }
 
 int factorize(hss_s* h, int prec, cudaStream_t st) {
@@ -729,7 +731,7 @@ int solve_levels(hss_s* h, Factor<T>& f, T* x, int nc, int ld, cudaStream_t st, 
   const LaunchLog log{h, st, sizeof(T) == 4};
   auto level = [&](int l) {
     const LevelT<T>& P = f.lv[l];
-    return LevelOf<T>{P.n, P.b, P.c, P.M, P.Li};
+    return LevelOf<T>{P.n, P.b, P.c, P.M, P.Li, P.Fl};
   };
   // this lane's columns of a level's vectors
   auto yv = [&](int l) { return f.lv[l].yv + (long long)col0 * f.lv[l].n * f.lv[l].b; };

@@ -78,6 +78,8 @@ struct FxShape {
   long long sPA;
   int tiles_m, tiles_n, tiles;
   int components;
+  const int* skip;
+  int skip_stride;
 };
 
 HSS_DEVINL uint32_t smem_of(const void* p) {
@@ -375,6 +377,7 @@ fx_gemm_kernel(const __grid_constant__ FxShape s) {
   unsigned char* smB = sm + kDigits * kRows * kPitch;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const long long z = blockIdx.x / s.tiles;
+  if (s.skip && s.skip[z * s.skip_stride]) return;
   int t = (int)(blockIdx.x % s.tiles), tm, tn;
   if (s.lower) {   // row block tm has the column blocks that start at or left of its last row
     tm = 0;
@@ -572,6 +575,7 @@ fx_skinny_kernel(const __grid_constant__ FxShape s) {
   for (int b = 0; b < NB; ++b) res[b] = 0.0;
   chain_wait();
   chain_release();
+  if (s.skip && s.skip[z * s.skip_stride]) return;
 
   for (int kt = 0; kt < s.K; kt += kGroup * TEAMS) {
     const int kg = kt + kGroup * team, ke = min(s.K, kg + kGroup), kw = kg + 32 * w;
@@ -805,9 +809,9 @@ cudaError_t fx_allow_smem(const void* kernel, int bytes) {
 cudaError_t fx_gemm(int m, int n, int K, const FxOperand& a, const FxOperand& b, double alpha,
                     double beta, const double* Cin, int ldcin, long long sCin, double* C, int ldc,
                     long long sC, int batch, bool lower, double* PA, int ldpa, long long sPA,
-                    cudaStream_t st, bool components) {
+                    cudaStream_t st, bool components, const int* skip, int skip_stride) {
   FxShape s{m, n, K, a.p2 ? K / 2 : K, a, b, alpha, beta, Cin ? Cin : C, ldcin, sCin, C, ldc, sC, lower ? 1 : 0,
-            PA, ldpa, sPA, 0, 0, 0, components ? 1 : 0};
+            PA, ldpa, sPA, 0, 0, 0, components ? 1 : 0, skip, skip_stride};
   // Narrow products (B's inner index contiguous).  Up to 8 columns fx_skinny_kernel is
   // the faster one at every size (512 x 512, 512 nodes: 481 against 506 us; 128 nodes:
   // 128 against 150; 128 x 128, 8 nodes: 6.2 against 10.5).  With 9 to 16 it wins while

@@ -21,11 +21,13 @@ struct FxOperand {
 // (z & 1) m of parent block z / 2.  Cin may be C.  components: every element
 // within about the bound of a DFMA chain, K 2^-53 Σ|a||b|; else (Householder
 // transformations) within K 2^-58.5 of the largest |a| times the largest |b| of its row
-// and column in each 128 inner indices.
+// and column in each 128 inner indices.  skip (may be null): problem z is left out where
+// skip[z skip_stride] is not zero, its C as it was.
 cudaError_t fx_gemm(int m, int n, int K, const FxOperand& a, const FxOperand& b, double alpha,
                     double beta, const double* Cin, int ldcin, long long sCin, double* C, int ldc,
                     long long sC, int batch, bool lower, double* PA, int ldpa, long long sPA,
-                    cudaStream_t st, bool components = true);
+                    cudaStream_t st, bool components = true, const int* skip = nullptr,
+                    int skip_stride = 0);
 
 // opts a kernel into `bytes` of dynamic shared memory, once per device and kernel
 cudaError_t fx_allow_smem(const void* kernel, int bytes);
