@@ -43,8 +43,7 @@ HSS_DEVINL void factor32(double* S, double* X, int o, double (*col)[64], double 
       double inv = 0.0, s = 0.0;
       if (d > 0.0) {
         inv = inv_sqrt(d);
-        s = d * inv;
-        s = fma(fma(-s, s, d), 0.5 * inv, s);
+        s = sqrt_from(d, inv);
       } else if (lane == 0) {
         report_failure(status, -3 /*NOT_SPD*/, level, node, col0 + o + j);
       }

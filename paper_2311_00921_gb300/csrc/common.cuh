@@ -54,8 +54,9 @@ HSS_DEVINL void report_failure(int* status, int code, int level, int node, int c
 }
 
 // 1 / sqrt(d), d > 0: y0 from FP32 on d scaled to [1, 4) by a power of four, then
-// y = y0 + y0 e (1/2 + 3/8 e), e = 1 - d y0² (Newton's iteration with the second
-// term of the series kept): the estimate's 2^-22 becomes 2^-63 before rounding.
+// y = y0 + y0 e (1/2 + 3/8 e), e = 1 - d y0² (Householder's iteration of third order,
+// the binomial series of (1 - e)^(-1/2) up to e²): the estimate's 2^-22 becomes 2^-63
+// before rounding.  Denormals, infinities and NaN take CUDA's square root and division.
 HSS_DEVINL double inv_sqrt(double d) {
   const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
   if (ex == 0 || ex == 0x7ff) return 1.0 / sqrt(d);
@@ -68,8 +69,16 @@ HSS_DEVINL double inv_sqrt(double d) {
   return __hiloint2double(__double2hiint(y) - (p << 20), __double2loint(y));
 }
 
-// 1 / d, d > 0, the same way: y = y0 (1 + e + e²), e = 1 - d y0, y0 the FP32 reciprocal
-// of d scaled to [1, 2)
+// sqrt(d), d > 0, from inv = inv_sqrt(d): d inv and one step of Heron's (Newton's)
+// iteration with the reciprocal at hand; infinity for infinity
+HSS_DEVINL double sqrt_from(double d, double inv) {
+  const double s = d * inv;
+  return inv == 0.0 ? d : fma(fma(-s, s, d), 0.5 * inv, s);
+}
+
+// 1 / d, d > 0: y = y0 (1 + e + e²), e = 1 - d y0, y0 the FP32 reciprocal of d scaled to
+// [1, 2) (Householder's iteration of third order, the geometric series up to e²).
+// Results near the ends of the range take CUDA's division.
 HSS_DEVINL double inv_pos(double d) {
   const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
   if (ex < 32 || ex > 0x7ff - 32) return 1.0 / d;

@@ -46,9 +46,7 @@ HSS_DEVINL void reflector(double alpha, double sigma, double* beta, double* tau,
     return;
   }
   const double s = fma(alpha, alpha, sigma), inv = inv_sqrt(s), aa = fabs(alpha);
-  double nrm = s * inv;
-  nrm = fma(fma(-nrm, nrm, s), 0.5 * inv, nrm);
-  const double sc = inv_pos(aa + nrm);
+  const double nrm = sqrt_from(s, inv), sc = inv_pos(aa + nrm);
   *beta = alpha >= 0.0 ? -nrm : nrm;
   *tau = fma(aa, inv, 1.0);
   *scale = alpha >= 0.0 ? sc : -sc;
