@@ -111,8 +111,10 @@ typedef enum { HSS_RESIDUAL_FP64 = 0, HSS_RESIDUAL_PAIR32 = 1 } hss_residual;
 
 /* Method of the basis completion (Eq. 2-3); both give the same V, T and L_B up
  * to rounding (the Householder QL with LAPACK's dlarfg signs).
- * HSS_BASIS_HOUSEHOLDER (default): the Householder kernel, one CTA per node
- * with a CTA-wide reduction per column.
+ * HSS_BASIS_HOUSEHOLDER (default): Householder QL.  Low ranks in one kernel, one CTA
+ * per node; FP64 above rank 16, FP32 above rank 128 (from rank 64 on levels of at least
+ * 152 nodes of order above 256) as panels of 16 or 32 columns, one CTA per node, with
+ * the later columns' updates and the factor T as products over the level.
  * HSS_BASIS_CHOLQR: Cholesky QR twice of the reversed basis as level-wide
  * products, then the Householder vectors reconstructed from the orthonormal
  * factor by an unpivoted LU of its top block (one CTA per node); nodes whose
@@ -123,13 +125,15 @@ typedef enum { HSS_BASIS_HOUSEHOLDER = 0, HSS_BASIS_CHOLQR = 1,
                HSS_BASIS_AUTO = 2 /* the choice of hss_tune, else HOUSEHOLDER */ } hss_basis_method;
 
 /* Schedule of the solve's upper levels (the levels of at most 64 nodes above
- * the leaves).  HSS_SCHEDULE_ASYNC: one launch per direction for all of them,
- * with no barrier between levels (asynchronous execution of the tree, Sec. 4.2):
- * going up, the CTA that finishes the second child of a node goes on with the
- * node; going down, a cooperative launch in which each node waits for its
- * parent's ready flag (a bounded wait, see wait_budget; an expired wait makes
- * the solve report HSS_ERR_TIMEOUT).  HSS_SCHEDULE_LEVELS: one launch per level
- * and direction.  Both give the same result. */
+ * the leaves), for ranks up to 16 in FP64 and up to 32 in the mixed modes.  Higher
+ * ranks have one schedule, products over a whole level, and this option, like the
+ * tuner's staging, changes nothing there.
+ * HSS_SCHEDULE_ASYNC: one launch per direction for all of them, with no barrier
+ * between levels (asynchronous execution of the tree, Sec. 4.2): going up, the CTA
+ * that finishes the second child of a node goes on with the node; going down, a
+ * cooperative launch in which each node waits for its parent's ready flag (a bounded
+ * wait, see wait_budget; an expired wait makes the solve report HSS_ERR_TIMEOUT).
+ * HSS_SCHEDULE_LEVELS: one launch per level and direction.  Both give the same result. */
 typedef enum { HSS_SCHEDULE_ASYNC = 0, HSS_SCHEDULE_LEVELS = 1,
                HSS_SCHEDULE_AUTO = 2 /* the choices of hss_tune (schedule and the sweeps'
                                         panel staging), else ASYNC */ } hss_schedule;
@@ -140,8 +144,9 @@ typedef struct {
   double ir_tol;       /* stop when every column has ‖b - A x‖₂ / ‖b‖₂ <= ir_tol */
   int32_t residual;    /* hss_residual (mixed modes) */
   int32_t basis;       /* hss_basis_method: how the basis completion is computed */
-  int64_t wait_budget; /* polls a device-side wait (tensor-core pipeline, ready flags of
-                          the solve) makes before it gives up and the call reports
+  int64_t wait_budget; /* polls a device-side wait (tensor-core pipeline; ready flags of
+                          the solve's HSS_SCHEDULE_ASYNC, which only the ranks given
+                          there have) makes before it gives up and the call reports
                           HSS_ERR_TIMEOUT (at the next synchronizing call); 0 = the
                           default, 2^24 polls.  A negative value makes
                           every such wait give up at once: a way to exercise the failure
@@ -258,7 +263,7 @@ int hss_matvec_noalloc(const hss_shape* shape, const double* D, const double* U,
  * panel width of the Householder basis kernel (16 or 32 columns: the wider
  * panel holds more of the basis in registers, the narrower one lets two CTAs
  * share an SM), the schedule of the solve's upper levels, the panel staging of
- * the solve's sweep kernels (0 = the largest shared-memory panels, 1 = the
+ * the solve's per-node sweep kernels (0 = the largest shared-memory panels, 1 = the
  * panels that let the fewest waves of CTAs cover a level), the refinement
  * lanes of a mixed solve, and the measured times of the chosen configuration. */
 typedef struct {
@@ -283,11 +288,12 @@ typedef struct {
  * CUDA events on `stream` -- each basis method (the Householder one with each
  * panel width its arithmetic has) on hss_factorize, each pair of
  * solve schedule and sweep panel staging on hss_solve of min(nrhs, 16)
- * columns of a fixed test vector -- best of two runs each, and keeps the
+ * columns of a fixed test vector (above the ranks that have these two options,
+ * one measurement, in solve_ms_by_config[0][0]) -- best of two runs each, and keeps the
  * fastest; later hss_factorize calls with basis = HSS_BASIS_AUTO or schedule =
  * HSS_SCHEDULE_AUTO use them.  cache_path (may be NULL): a text file of
- * earlier choices, one line per key (device name, precision, residual, n,
- * leaf, rank, levels, columns); a matching line is used instead of measuring,
+ * earlier choices, one line per key (version of the candidates, device name,
+ * precision, residual, n, leaf, rank, levels, columns); a matching line is used instead of measuring,
  * and a new measurement is appended.  Leaves the object factorized with the
  * chosen configuration.  Allocates two n x 16 vectors for the duration of the
  * call.  Synchronous.  out may be NULL.  Errors: as hss_factorize and

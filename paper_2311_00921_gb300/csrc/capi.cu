@@ -38,6 +38,8 @@ constexpr int kTreeRank = 16;     // FP64 solves up to this rank run on the per-
 constexpr int kTreeRank32 = 32;   // FP32 sweeps up to this one (see solve_levels)
 constexpr int kFuseNodes = 64;    // levels up to this many nodes apply Q inside the sweep kernel
 constexpr int kTreeTop = 6;       // levels 1 .. 6 (<= 64 nodes): one tree launch per direction
+constexpr int kTuneVersion = 2;   // of the tuner's candidates: raised when their kernels change,
+                                  // so that choices cached before are measured again
 
 template <typename T>
 struct LevelT {
@@ -1458,8 +1460,8 @@ int hss_tune(hss_t h, const hss_options* opt, int32_t nrhs, const char* cache_pa
     int q = 0;
     for (const char* c = prop.name; *c && q < 255; ++c) dev[q++] = (*c == ' ' ? '_' : *c);
     dev[q] = 0;
-    snprintf(key, sizeof key, "%s p%d res%d n%d leaf%d rank%d L%d cols%d", dev, opt->precision,
-             opt->residual, h->n_user, h->leaf, h->rank, h->L, nc);
+    snprintf(key, sizeof key, "v%d %s p%d res%d n%d leaf%d rank%d L%d cols%d", kTuneVersion, dev,
+             opt->precision, opt->residual, h->n_user, h->leaf, h->rank, h->L, nc);
   }
   bool found = false;
   if (cache_path) {
@@ -1557,6 +1559,11 @@ int hss_tune(hss_t h, const hss_options* opt, int32_t nrhs, const char* cache_pa
       h->tuned = 0;
     }
     best.solve_ms = 1e30;
+    // above the per-node kernels' ranks the sweeps have one schedule and no staging
+    // (solve_levels): one measurement, listed under the default pair
+    const bool per_node = h->rank <= (o.precision == HSS_FP64 ? kTreeRank : kTreeRank32);
+    const int last_sched = per_node ? HSS_SCHEDULE_LEVELS : HSS_SCHEDULE_ASYNC;
+    const int last_staging = per_node ? 1 : 0;
     // refinement lanes: two only where they apply (a mixed factor with the FP64
     // residual and at least two columns)
     const int max_lanes =
@@ -1564,9 +1571,8 @@ int hss_tune(hss_t h, const hss_options* opt, int32_t nrhs, const char* cache_pa
     for (int lanes = 1; rc == HSS_OK && lanes <= max_lanes; ++lanes) {
       h->ir_lanes = lanes;
       double lane_best = 1e30;
-      for (int sched = HSS_SCHEDULE_ASYNC; rc == HSS_OK && sched <= HSS_SCHEDULE_LEVELS;
-           ++sched) {
-        for (int stg = 0; rc == HSS_OK && stg <= 1; ++stg) {
+      for (int sched = HSS_SCHEDULE_ASYNC; rc == HSS_OK && sched <= last_sched; ++sched) {
+        for (int stg = 0; rc == HSS_OK && stg <= last_staging; ++stg) {
           h->schedule = sched;
           h->staging = stg;
           double ms = 0.0;
