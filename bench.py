@@ -210,6 +210,32 @@ KERNEL_SOURCES = {"tc_gemm": "tc_gemm_kernel", "tc_syr2k": "tc_gemm_kernel",
                   "trsv_bwd": "trsv_bwd_kernel", "other": "logdet_reduce_kernel",
                   "pair_gemm": "df_gemm_kernel", "basis_gemm": "basis_gemm_kernel",
                   "basis_node": "recon_lu_kernel"}
+# What runs instead at a given precision and above a given rank (the library's dispatch:
+# sliced FP64 products at every rank; panels and level-wide sweeps above 16 in FP64, 32 in
+# FP32).  Where a class has several kernels the first has the largest launches.
+KERNELS_ABOVE = {
+    "f64": ((0, {"gemm": ("fx_gemm_kernel",), "gemm_skinny": ("fx_gemm_kernel", "fx_skinny_kernel"),
+                 "syr2k": ("fx_gemm_kernel",), "pchol": ("chol64_kernel",)}),
+            (16, {"ql": ("ql_panel_kernel",), "basis_node": ("ql_tblock_kernel",),
+                  "trsv_fwd": ("fx_gemm_kernel", "fx_skinny_kernel"),
+                  "trsv_bwd": ("fx_gemm_kernel", "fx_skinny_kernel")})),
+    "f32": ((32, {"gemm_skinny": ("narrow32_kernel",), "trsv_fwd": ("narrow32_kernel",),
+                  "trsv_bwd": ("narrow32_kernel",)}),
+            (63, {"ql": ("ql_basis_kernel", "ql_panel_kernel")}),
+            (128, {"ql": ("ql_panel_kernel",), "basis_node": ("ql_tblock_kernel",)}))}
+SLICED_MMAS = 36   # FP16 MMAs per product of the sliced FP64 kernels
+
+
+def kernels_of(kind, prec, rank):
+    """The kernels behind a class of the tracer; rank None: KERNEL_SOURCES alone."""
+    names = (KERNEL_SOURCES[kind],)
+    if rank is not None:
+        for above, table in KERNELS_ABOVE.get(prec, ()):
+            if rank > above:
+                names = table.get(kind, names)
+    return names
+
+
 # pair-of-FP32 arithmetic: 12 FP32 instructions per multiply-add (2 flops) plus a
 # 3-instruction renormalisation every 4 terms
 PAIR_OPS_PER_FLOP = 12.75 / 2
@@ -310,7 +336,9 @@ def measured_peaks(torch):
     return peaks
 
 
-PEAK_SOURCE = {"pair32": "cuBLAS SGEMM 8192^3 without TF32 (FP32 SIMT) measured in this run, "
+PEAK_SOURCE = {"sliced64": "cuBLAS BF16 GEMM 8192^3 measured in this run, / 36: an FP64 product by "
+                           "exact slicing is 36 FP16 MMAs (the rate of BF16)",
+               "pair32": "cuBLAS SGEMM 8192^3 without TF32 (FP32 SIMT) measured in this run, "
                          "/ 6.375: the pair arithmetic spends 12.75 FP32 instructions per "
                          "multiply-add",
                "f64": "cuBLAS DGEMM 8192^3 (FP64 pipe) measured in this run",
@@ -362,9 +390,11 @@ PREC_LABEL = {"f64": "FP64", "f32": "FP32", "tf32": "TF32 x3", "bf16": "BF16 x3"
               "pair32": "pair-of-FP32"}
 
 
-def roofline_of(tr, peaks, steps, prec_mode="fp64", overlapped=None, overlapped_steps=None):
+def roofline_of(tr, peaks, steps, prec_mode="fp64", overlapped=None, overlapped_steps=None,
+                rank=None):
     """Roofline of the dominant kernel class of trace `tr` (a serialized pass:
-    every logged duration is the kernel's own).  `overlapped` is the trace of the
+    every logged duration is the kernel's own), its kernels those of a matrix of
+    rank `rank`.  `overlapped` is the trace of the
     run as timed (basis chain concurrent on a second stream), reported beside it."""
     dom = max(tr, key=lambda k: tr[k][0])
     dms, dn, dfl = tr[dom]
@@ -372,10 +402,15 @@ def roofline_of(tr, peaks, steps, prec_mode="fp64", overlapped=None, overlapped_
     if kind.startswith("tc_"):
         prec = prec_mode   # tensor-core kernels: the MMA input type's peak
     achieved = dfl / (dms / 1e3) / 1e12 if dms > 0 else 0.0
-    kname = KERNEL_SOURCES[kind]
+    names = kernels_of(kind, prec, rank)
+    kname = names[0]
     peak = peaks.get(prec) if peaks else None
+    if kname.startswith("fx_"):
+        peak, peak_key = peaks["bf16"] / SLICED_MMAS if peaks else None, "sliced64"
+    else:
+        peak_key = prec
     if kind == "pair_gemm":
-        prec = "pair32"
+        prec = peak_key = "pair32"
         peak = peaks["f32"] / PAIR_OPS_PER_FLOP if peaks else None
     total = sum(v[0] for v in tr.values())
     traffic = traffic_record(kname, prec)
@@ -384,8 +419,8 @@ def roofline_of(tr, peaks, steps, prec_mode="fp64", overlapped=None, overlapped_
            "traffic": traffic[0] if traffic else None,
            "traffic_launch": traffic[1] if traffic else None,
            "traffic_algorithmic_bytes": traffic[2] if traffic else None,
-           "kernel": f"{kname} ({PREC_LABEL.get(prec, prec)})",
-           "peak_source": PEAK_SOURCE.get(prec),
+           "kernel": f"{', '.join(names)} ({PREC_LABEL.get(prec, prec)})",
+           "peak_source": PEAK_SOURCE.get(peak_key),
            "timing": "serialized pass (basis chain on the main stream), CUDA events per launch",
            "kernel_ms_per_launch": dms / max(1, dn), "kernel_launches_per_step": dn / steps,
            "kernel_share": dms / total,
@@ -556,7 +591,7 @@ def run_ours(args):
             v64["headline_speedup_vs_fp64"] = v64["ms_per_step"] / ms_step
             v64["roofline"] = roofline_of(ser64["trace"], peaks, min(args.steps, 3), "fp64",
                                           overlapped=g64["trace"],
-                                          overlapped_steps=g64["trace_steps"])
+                                          overlapped_steps=g64["trace_steps"], rank=w.rank)
             fp64 = v64
 
     e2e = None
@@ -603,7 +638,7 @@ def run_ours(args):
                "fp64": fp64, "variants": variants,
                "roofline": roofline_of(ser["trace"], peaks, nser, prec,
                                        overlapped=traced["trace"],
-                                       overlapped_steps=min(args.steps, 5)),
+                                       overlapped_steps=min(args.steps, 5), rank=w.rank),
                "cpu_baseline": cpu, "e2e": e2e, "clocks": head["clocks"],
                "autotune": tuning, "precision_choice": choice,
                "gpu_launches": head["launches"]}
