@@ -43,8 +43,8 @@
 // issues MMAs.
 #include <stdint.h>
 
-#include <map>
 #include <mutex>
+#include <set>
 #include <utility>
 
 #include "common.cuh"
@@ -793,16 +793,15 @@ cudaError_t launch_modes(FxShape& s, int batch, cudaStream_t st) {
 
 cudaError_t fx_allow_smem(const void* kernel, int bytes) {
   static std::mutex mu;
-  static std::map<std::pair<int, const void*>, cudaError_t> memo;
+  static std::set<std::pair<int, const void*>> memo;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> g(mu);
   const auto key = std::make_pair(dev, kernel);
-  const auto it = memo.find(key);
-  if (it != memo.end()) return it->second;
+  if (memo.count(key)) return cudaSuccess;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  memo[key] = e;
+  if (e == cudaSuccess) memo.insert(key);   // a failure is tried, and reported, again
   return e;
 }
 
