@@ -96,6 +96,27 @@ HSS_DEVINL T warp_sum(T v) {
   return v;
 }
 
+// Sum over the 32 lanes of acc[k] lands in lane k (k < NV; NV = 16 or 32):
+// a transposing butterfly, NV - 1 (+ NV for NV = 16) shuffles instead of NV * 5.
+template <typename T, int NV>
+HSS_DEVINL T warp_transpose_reduce(T (&acc)[NV], int lane) {
+  if (NV == 16) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
+  }
+#pragma unroll
+  for (int s = NV / 2; s >= 1; s >>= 1) {
+    const bool upper = (lane & s) != 0;
+#pragma unroll
+    for (int i = 0; i < s; ++i) {
+      const T send = upper ? acc[i] : acc[i + s];
+      const T keep = upper ? acc[i + s] : acc[i];
+      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+    }
+  }
+  return acc[0];
+}
+
 // block-wide sum over blockDim.x threads (multiple of 32); `red` holds >= 32
 // elements of shared scratch.  Every thread gets the total.
 template <typename T>

@@ -16,26 +16,6 @@
 
 namespace {
 
-// Sum over the 32 lanes of acc[k] lands in lane k (k < NV; NV = 16 or 32).
-template <typename T, int NV>
-HSS_DEVINL T transpose_reduce(T (&acc)[NV], int lane) {
-  if (NV == 16) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
-  }
-#pragma unroll
-  for (int s = NV / 2; s >= 1; s >>= 1) {
-    const bool upper = (lane & s) != 0;
-#pragma unroll
-    for (int i = 0; i < s; ++i) {
-      const T send = upper ? acc[i] : acc[i + s];
-      const T keep = upper ? acc[i + s] : acc[i];
-      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-    }
-  }
-  return acc[0];
-}
-
 // reflector of (alpha, x), |x|² = sigma (LAPACK's dlarfg signs): beta, tau and the
 // factor that turns x into v below its unit entry
 HSS_DEVINL void reflector(double alpha, double sigma, double* beta, double* tau, double* scale) {
@@ -116,7 +96,7 @@ ql_panel_kernel(const T* __restrict__ Bb, T* __restrict__ Wb, T* __restrict__ Vb
 #pragma unroll
       for (int k = jj; k < NB; ++k) g[k] = fma(a, x[s][k], g[k]);
     }
-    const T gw = transpose_reduce<T, NB>(g, lane);
+    const T gw = warp_transpose_reduce<T, NB>(g, lane);
     if (lane < NB) red[buf][wid][lane] = gw;
     __syncthreads();
     T gk = T(0);   // Σ_{i>j} x_ij x_ik for k = lane
@@ -191,7 +171,7 @@ ql_panel_kernel(const T* __restrict__ Bb, T* __restrict__ Wb, T* __restrict__ Vb
         else if (c2 != c) g[q] = fma(x[s][q - c], x[s][c2], g[q]);
       }
     }
-    const T gw = transpose_reduce<T, NB>(g, lane);
+    const T gw = warp_transpose_reduce<T, NB>(g, lane);
     if (lane < c) Gs[wid][c][lane] = gw;
     else if (lane < NB && c2 != c) Gs[wid][c2][lane - c] = gw;
   }

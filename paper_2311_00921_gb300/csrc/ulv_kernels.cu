@@ -9,8 +9,7 @@
 //                         partial-Cholesky (Alg. 2), for every node of a
 //                         level: POTRF of the diagonal block and TRSM of the rows
 //                         below it; the trailing SYRK is a level-wide launch
-//                         (gemm.cu).  With c = b it is the panel of the root
-//                         Cholesky (the last step of Alg. 2).
+//                         (gemm.cu).  FP32 factors only (FP64: chol64.cu).
 //  * scatter_ss_kernel -- the merge (Alg. 2) as its own pass: Â^SS of each node
 //                         into its parent's diagonal block.  Used only where a
 //                         level eliminates nothing (rank = block order); otherwise
@@ -38,27 +37,6 @@ constexpr int NT = 256;
 constexpr int NB = 32;   // panel width of the blocked Cholesky / triangular solves
 
 // ------------------------------------------------------------------ QL
-// Sum over the 32 lanes of acc[k] lands in lane k (k < NV; NV = 16 or 32):
-// a transposing butterfly, NV - 1 (+ NV for NV = 16) shuffles instead of NV * 5.
-template <typename T, int NV>
-HSS_DEVINL T warp_transpose_reduce(T (&acc)[NV], int lane) {
-  if (NV == 16) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
-  }
-#pragma unroll
-  for (int s = NV / 2; s >= 1; s >>= 1) {
-    const bool upper = (lane & s) != 0;
-#pragma unroll
-    for (int i = 0; i < s; ++i) {
-      const T send = upper ? acc[i] : acc[i + s];
-      const T keep = upper ? acc[i + s] : acc[i];
-      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-    }
-  }
-  return acc[0];
-}
-
 // CTA-level product O(q, c) = Σ_{i >= i0} Pt(q, i) A(i, c) for q < NBP and the
 // ncols columns of A (column c at A + c * lda): the panel's reflectors (Pt,
 // transposed in shared memory with row pitch NBP + 1) against 64-row slabs of A
@@ -413,11 +391,7 @@ HSS_DEVINL T reg_select(const T (&a)[NB], int i) {
 // separate level-wide SYRK.  Warp 0 factors the kb x kb diagonal block in
 // registers (lane i holds row i, the pivot and the column entries travel by
 // shuffles), then every thread solves rows of X L_11ᵀ = M_21 below it in
-// registers against the block kept in shared memory.  With several row splits
-// (a lone node, e.g. the root, whose row solves would otherwise queue on one
-// SM's FP64 pipe) each CTA factors the diagonal block itself and solves its own
-// share of the rows; split 0 alone writes the block, the log-det and a failure.
-// The node's log-det slot gets (or, with accumulate, adds) 2 Σ log L_jj.
+// registers against the block kept in shared memory.  The node's log-det slot gets (or, with accumulate, adds) 2 Σ log L_jj.
 template <typename T>
 __global__ void __launch_bounds__(NT)
 chol_panel_kernel(T* Mb, int ldm, long long sM, int rows, int kb, double* logdet_part, int level,
@@ -426,7 +400,6 @@ chol_panel_kernel(T* Mb, int ldm, long long sM, int rows, int kb, double* logdet
   __shared__ T dinv[NB];
   __shared__ int fail;
   const int node = blockIdx.x;
-  const bool lead = blockIdx.y == 0;
   T* M = Mb + (long long)node * sM;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (wid == 0) {
@@ -453,20 +426,20 @@ chol_panel_kernel(T* Mb, int ldm, long long sM, int rows, int kb, double* logdet
     }
     if (lane == 0) fail = bad >= 0;
     if (bad >= 0) {
-      if (lane == 0 && lead)
+      if (lane == 0)
         report_failure(status, -3 /*NOT_SPD*/, level, node0 + node, col0 + bad);
     } else {
 #pragma unroll
       for (int t = 0; t < NB; ++t)
         if (lane < kb && t <= lane) {
-          if (lead) M[lane + (long long)t * ldm] = a[t];
+          M[lane + (long long)t * ldm] = a[t];
           Ls[lane][t] = a[t];
         }
       const T dg = reg_select(a, lane);
       if (lane < kb) dinv[lane] = T(1) / dg;
       double ld = lane < kb ? log((double)dg) : 0.0;
       ld = warp_sum(ld);
-      if (lane == 0 && logdet_part && lead) {
+      if (lane == 0 && logdet_part) {
         if (accumulate)
           logdet_part[node] += 2.0 * ld;
         else
@@ -476,10 +449,7 @@ chol_panel_kernel(T* Mb, int ldm, long long sM, int rows, int kb, double* logdet
   }
   __syncthreads();
   if (fail) return;
-  // this split's rows: [kb + per y, kb + per (y + 1))
-  const int per = (rows - kb + gridDim.y - 1) / gridDim.y;
-  const int i0 = kb + per * blockIdx.y, i1 = min(rows, i0 + per);
-  for (int i = i0 + tid; i < i1; i += NT) {
+  for (int i = kb + tid; i < rows; i += NT) {
     T x[NB];
 #pragma unroll
     for (int t = 0; t < NB; ++t) x[t] = t < kb ? M[i + (long long)t * ldm] : T(0);
@@ -1238,12 +1208,10 @@ cudaError_t launch_ql_basis(const T* Bsrc, int ldb_src, long long sB, T* V, long
 template <typename T>
 cudaError_t launch_chol_panel(T* M, int ldm, long long sM, int rows, int kb, double* logdet_part,
                               int level, int node0, int col0, int* status, int nodes,
-                              bool accumulate, cudaStream_t st, int splits) {
-  if (kb < 1 || kb > NB || rows < kb || splits < 1 || splits > 65535)
-    return cudaErrorInvalidValue;
-  chol_panel_kernel<T><<<dim3(nodes, splits), NT, 0, st>>>(M, ldm, sM, rows, kb, logdet_part,
-                                                           level, node0, col0, status,
-                                                           accumulate ? 1 : 0);
+                              bool accumulate, cudaStream_t st) {
+  if (kb < 1 || kb > NB || rows < kb) return cudaErrorInvalidValue;
+  chol_panel_kernel<T><<<nodes, NT, 0, st>>>(M, ldm, sM, rows, kb, logdet_part, level, node0, col0,
+                                             status, accumulate ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -1482,8 +1450,6 @@ void launch_logdet_reduce(const double* part, int n, double* out, cudaStream_t s
                                          int, const T*, int, long long, const T*, long long,      \
                                          const T*, long long, int, int, cudaStream_t, int);       \
   template size_t ql_smem<T>(int, int, int);                                                     \
-  template cudaError_t launch_chol_panel<T>(T*, int, long long, int, int, double*, int, int, int,\
-                                            int*, int, bool, cudaStream_t, int);                  \
   template cudaError_t launch_scatter_ss<T>(const T*, int, long long, int, int, T*, int,           \
                                             long long, int, cudaStream_t);                       \
   template cudaError_t launch_tree_fwd<T>(const TreeLevels<T>&, int, int, int, int, int, int*,    \
@@ -1494,3 +1460,5 @@ void launch_logdet_reduce(const double* part, int n, double* out, cudaStream_t s
   template bool tree_fits<T>(int, int, int);
 INST(double)
 INST(float)
+template cudaError_t launch_chol_panel<float>(float*, int, long long, int, int, double*, int, int, int,
+                                              int*, int, bool, cudaStream_t);
