@@ -719,14 +719,18 @@ int sweep_root(hss_s* h, Factor<T>& f, T* v0, int nc, int col0, cudaStream_t st)
 }
 
 // The ULV sweeps as products over whole levels: Q by three, each triangular sweep by
-// two per 128 eliminated columns (chol64.cuh).  A node's sweep in one CTA is in FP64
-// bound by that SM's pipe, 540 us a level and direction at rank 128 with 16 columns
-// (78 us at rank 32 with one) against 50 us (25 us) for the products; up to rank
-// kTreeRank the per-node kernels, one launch for all upper levels, are as fast or
-// faster and stay.  In FP32 it is a chain of 32-column steps: rank 128, 16 columns,
-// 151 us a level and direction on average of N = 262144 against 71, rank 96, 3 columns,
-// 50 against 22.  The line is at rank 32 there: N = 16384, one column, 1.06 ms by the
-// tree kernels and 1.15 by products at rank 32, 1.24 and 1.16 at rank 48.
+// two per 128 eliminated columns and in FP64 two more, its correction (chol64.cuh).  A
+// node's sweep in one CTA is in FP64 bound by that SM's pipe, 540 us a level and
+// direction at rank 128 with 16 columns (78 us at rank 32 with one) against 50 us (25 us)
+// for the products, 13 to 18 % more with corrections that return at once.  Up to rank
+// kTreeRank the per-node kernels stay, one launch for all upper levels (leaf 64, rank 4,
+// five levels: 281 us a solve).  That holds for small leaves: the rule does not look at
+// the leaf, and levels of 512 x 512 leaves of rank 16 take 3.3 ms a solve in their CTAs,
+// where rank 48 takes 0.5 ms by products.  In FP32 the CTA's sweep is a chain of
+// 32-column steps: rank 128, 16 columns, 151 us a level and direction on average of
+// N = 262144 against 71, rank 96, 3 columns, 50 against 22.  The line is at rank 32
+// there: N = 16384, one column, 1.06 ms by the tree kernels and 1.15 by products at
+// rank 32, 1.24 and 1.16 at rank 48.
 template <typename T>
 int solve_levels(hss_s* h, Factor<T>& f, T* x, int nc, int ld, cudaStream_t st, int col0) {
   const int L = h->L;

@@ -34,7 +34,9 @@ cudaError_t launch_ql_tblocks(const T* G, T* Tm, int r, int nodes, cudaStream_t 
 // 3.1 ms, the levels above 2.2 -> 1.3 ms).  At lower ranks it gains on a level with more
 // nodes than SMs and more rows than a CTA has threads, where the one-CTA kernel runs in
 // several waves of two rows a thread (512 leaves of 512 x 128, 3.0 ms of the critical path:
-// the step 22.1 -> 21.0 ms).
+// the step 22.1 -> 21.0 ms; FP32 factor by one CTA a node and by panels, leaf x rank,
+// leaves: 300 x 64, 256: 3.18 and 3.02 ms; 512 x 64, 256: 5.02 and 4.75; 512 x 96, 256:
+// 6.72 and 6.40; 260 x 96, 512: 6.94 and 6.50; 300 x 127, 256: 7.26 and 6.73).
 template <typename T>
 bool ql_blocked(int b, int r, int nodes) {
   if (sizeof(T) == 8) return r > 16;

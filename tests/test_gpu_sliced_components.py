@@ -93,7 +93,10 @@ def test_denormal_rows():
 @pytest.mark.parametrize("peak", [1.0, 1000.0])
 def test_not_less_accurate_than_a_chain(leaf, nrhs, levels, peak):
     """Root-mean-square error against that of a sequential chain in FP64 (products
-    exact, one rounding a step), for uniform rows and for rows with a large diagonal."""
+    exact, one rounding a step), for uniform rows and for rows with a large diagonal.  The
+    sliced product rounds once per group of 128 indices: at most half the chain's error
+    from 256 indices on, which seven digits (2^-56 of the scales' product per index, as
+    much as the chain itself at these sizes) would not keep."""
     rng = _rng(leaf, nrhs, 4)
     nodes = 1 << levels
     D = rng.standard_normal((nodes, leaf, leaf))
@@ -105,7 +108,7 @@ def test_not_less_accurate_than_a_chain(leaf, nrhs, levels, peak):
     for k in range(leaf):
         chain = (chain + Dl[:, :, k, None] * xl[:, None, k, :]).astype(np.float64)
     rms = lambda v: float(np.sqrt(np.mean(((v - ref).astype(np.float64)) ** 2)))
-    assert rms(_product(D, x, levels)) <= rms(chain)
+    assert rms(_product(D, x, levels)) <= (0.5 if leaf >= 256 else 1.0) * rms(chain)
 
 
 @pytest.mark.parametrize("levels,leaf,rank", [(1, 96, 20), (2, 160, 40), (1, 256, 64), (2, 64, 32)])
