@@ -413,7 +413,8 @@ def roofline_of(tr, peaks, steps, prec_mode="fp64", overlapped=None, overlapped_
         prec = peak_key = "pair32"
         peak = peaks["f32"] / PAIR_OPS_PER_FLOP if peaks else None
     total = sum(v[0] for v in tr.values())
-    traffic = traffic_record(kname, prec)
+    # a sliced product's record is that of one class of launches
+    traffic = traffic_record(f"{kname}:{kind}" if kname.startswith("fx_") else kname, prec)
     out = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
            "frac": (achieved / peak) if peak else None,
            "traffic": traffic[0] if traffic else None,

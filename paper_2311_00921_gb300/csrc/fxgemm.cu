@@ -26,7 +26,10 @@
 // columns (a chain's bound K 2^-53 of them is 2^5 of the above), do without S
 // (components = false): the reflectors' unit entries and zeros would send up to 22 % of
 // their elements to the DFMA pipe.  Batch of ten: 11.4 ms without S, 13.9 ms with S
-// in all products, 12.0 ms so; D x of 512 leaves and 16 columns is 5 % slower with S.
+// in all products, 12.2 ms so; D x of 512 leaves and 16 columns is 5 % slower with S.
+// The merges' products, L_B (nearly diagonal) times couplings of a wide range, send 5 to
+// 30 % of their elements there: factor of the sphere workload's matrix, N = 262144, 52
+// ms without S and 57.7 with it, of random generators 52 and 53.
 // (Seven digits, whose error is 2^-56 of max|a| max|b|, are not enough: the solves of
 // kernel matrices lost a factor of three to five against the DFMA chain.)
 //
@@ -346,7 +349,10 @@ template <int NB, typename SA, typename SB>
 __device__ __noinline__ void small_sums(const SA& A, const SB& B, int k0, int k1, uint32_t which,
                                         double (&res)[NB][4]) {
   const int w = threadIdx.x >> 5;
-  if (__reduce_add_sync(0xffffffffu, __popc(which)) > 64 * NB) {
+  // of 128 NB: there 300 clocks a sum meet the chains' 8192 a fragment register (merges of
+  // real couplings: factor of the grid covariance, N = 65536, 21.3 ms with the line at
+  // half, 19.8 here)
+  if (__reduce_add_sync(0xffffffffu, __popc(which)) > 104 * NB) {
     plain_group<NB>(A, B, k0, k1, which, res);
     return;
   }
